@@ -120,15 +120,12 @@ typedef struct {
     int straggling;         /* Bohr straggling on/off                                     */
     int nuclear;            /* nuclear removal (1.2 %/cm x density) on/off                */
     int frac_bits;          /* fixed-point scale of deposits, 2^-frac_bits MeV (default 24) */
-    /* Autotuned launch: the first dose (or influence-matrix) call of a
-     * context times a few launch configurations on a sample of its
-     * histories (up to 24 per thread of the largest block, about 3.3e6 on
-     * 152 SMs); the choice is kept by the context and, for later contexts
-     * on the same device with the same grids, field devices and fixed launch
-     * options, by the process.  Results do not depend on the choice. */
-    int aggregate;          /* -1 autotuned, 0 plain atomics, 1 warp-aggregated atomics   */
-    int block_size;         /* 0 autotuned, else patient-kernel threads per block (multiple of 32, <= 896) */
-    int blocks_per_sm;      /* 0 autotuned                                                */
+    /* Launch configuration; results do not depend on it.  The defaults are
+     * one shape for every call (896 threads per SM, plain atomics, chunks of
+     * 32 histories). */
+    int aggregate;          /* -1 default, 0 plain atomics, 1 warp-aggregated atomics     */
+    int block_size;         /* 0 default, else patient-kernel threads per block (multiple of 32, <= 896) */
+    int blocks_per_sm;      /* 0 default                                                  */
     int chunk;              /* histories taken per warp refill (0 = default)              */
     vpmc_history_record* history_out;  /* device buffer or NULL                          */
     int64_t history_cap;    /* records for global history index < history_cap            */
@@ -155,7 +152,7 @@ typedef struct {
     int64_t histories, steps, errors;
     double e_in, e_dep, e_leak, e_rs, e_aperture, e_nuc;
     float ms;               /* device time of the transport launch(es), CUDA events */
-    int64_t launches;       /* kernels this call launched (autotuning included) */
+    int64_t launches;       /* kernels this call launched  */
     int64_t ovf_records;    /* influence matrix: deposits outside their column's dense box */
     int64_t steps_rs;       /* condensed-history steps in the range shifter (included in steps) */
     int64_t steps_aperture; /* condensed-history steps in the brass block (included in steps) */
@@ -179,7 +176,7 @@ typedef struct {
 } vpmc_csr;
 
 /* Fill opts with defaults: seed 1234, all physics on, frac_bits 24,
- * autotuned launch, no records, brass range rejection on, iteration cap
+ * default launch, no records, brass range rejection on, iteration cap
  * 200,000. */
 void vpmc_default_opts(vpmc_opts* opts);
 
@@ -243,7 +240,7 @@ vpmc_status vpmc_run_spots(vpmc_ctx* ctx, const vpmc_spot* spots, int n_spots, c
  * and the status rules (stats_out, and the latched status word read by the
  * next call on the same device) are those of vpmc_run_spots, with the plain
  * aperture only (opts->surrogate = 1 is VPMC_ERR_ARG); the launch
- * configuration is the context's tuned one (or opts') without autotuning. */
+ * configuration is the same. */
 vpmc_status vpmc_run_spots_noalloc(vpmc_ctx* ctx, const vpmc_spot* spots, int n_spots, const vpmc_scenario* scen,
                                    const vpmc_opts* opts, float* dose_dev, vpmc_stats* stats_out);
 

@@ -6,7 +6,6 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
-#include <mutex>
 #include <vector>
 
 #include "../../include/vpmc.h"
@@ -402,7 +401,7 @@ vpmc_status ensure_phase(vpmc_ctx* c, long long total, bool surrogate = false)
 // Enqueues the transport of histories [0, total) of p's items: batches of at
 // most phase_cap / n_rep histories, each the devices kernel then the patient
 // kernel (which takes n_rep copies of every survivor, one per scenario).
-vpmc_status enqueue_transport(vpmc_ctx* c, TransportParams p, long long total, const TuneResult& t)
+vpmc_status enqueue_transport(vpmc_ctx* c, TransportParams p, long long total, const LaunchShape& t)
 {
     if (p.n_rep < 1) p.n_rep = 1;
     const long long batch = c->phase_cap / p.n_rep;
@@ -450,156 +449,6 @@ vpmc_status enqueue_transport(vpmc_ctx* c, TransportParams p, long long total, c
         c->launches += 3;
     }
     return VPMC_OK;
-}
-
-float time_launch(vpmc_ctx* c, cudaError_t (*fn)(const TransportParams&, int, int, cudaStream_t),
-                  const TransportParams& p, int block, int kernels)
-{
-    cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), c->stream);
-    cudaEventRecord(c->ev0, c->stream);
-    cudaError_t e = fn(p, c->num_sms, block, c->stream);
-    cudaEventRecord(c->ev1, c->stream);
-    if (e != cudaSuccess || cudaEventSynchronize(c->ev1) != cudaSuccess) return 1e30f;
-    c->launches += kernels;
-    float ms = 0.0f;
-    cudaEventElapsedTime(&ms, c->ev0, c->ev1);
-    return ms;
-}
-
-// Chooses the two kernels' block sizes, warp aggregation and refill chunk by
-// timing launches over a prefix of the work (results are discarded; the
-// caller zeroes the scoring buffers afterwards).  The prefix gives every lane
-// of the largest block about 24 histories: in a launch of only a few
-// histories per lane the tail (the last long histories of each warp) decides
-// the time and favours small blocks, which lose on long launches (13-scenario
-// head set: 768 threads chosen on 4 histories per lane, 4.7 % slower than the
-// 896 chosen on 24).
-vpmc_status autotune(vpmc_ctx* c, TransportParams p, TuneResult* out, const vpmc_opts& o)
-{
-    const long long sample = std::min<long long>(p.total, (long long)c->num_sms * patient_max_block() * 24);
-    TuneResult best;
-    best.valid = true;
-    if (o.block_size) best.block = o.block_size;
-    if (o.aggregate >= 0) best.aggregate = o.aggregate;
-    if (o.chunk) best.chunk = o.chunk;
-    if (sample <= 0) { *out = best; return VPMC_OK; }
-    p.records = nullptr;
-    p.rec_cap = 0;
-    p.hist_begin = 0;
-    p.total = sample;
-    p.surrogate = 0;            // timed on the plain beam-line path
-    p.chunk = best.chunk;
-    p.aggregate = best.aggregate;
-    // devices kernel block size (its output is identical for every choice)
-    float t_best = 1e30f;
-    for (int rep = 0; rep < 2; ++rep)
-        for (int block : {384, 512, 640}) {
-            CUDA_TRY(cudaMemsetAsync(c->d_phase_count, 0, sizeof(unsigned long long), c->stream));
-            vpmc_status st = reset_counters(c);
-            if (st != VPMC_OK) return st;
-            const float ms = time_launch(c, launch_devices, p, block, 2);
-            if (rep == 1 && ms < t_best) { t_best = ms; best.dev_block = block; }
-        }
-    // patient kernel on the histories the last devices launch handed over
-    t_best = 1e30f;
-    for (int rep = 0; rep < 2; ++rep)
-        for (int block : {512, 640, 768, 896})
-            for (int agg : {0, 1})
-                for (int chunk : {32, 128}) {
-                    if (block > patient_max_block() || (o.block_size && block != o.block_size)) continue;
-                    if (o.aggregate >= 0 && agg != o.aggregate) continue;
-                    if (o.chunk && chunk != o.chunk) continue;
-                    p.aggregate = agg;
-                    p.chunk = chunk;
-                    vpmc_status st = reset_counters(c);
-                    if (st != VPMC_OK) return st;
-                    const float ms = time_launch(c, launch_patient, p, block, 1);
-                    if (rep == 1 && ms < t_best) {
-                        t_best = ms;
-                        best.block = block;
-                        best.aggregate = agg;
-                        best.chunk = chunk;
-                    }
-                }
-    *out = best;
-    return VPMC_OK;
-}
-
-// Process-wide cache of tuned launch configurations.  The launch choices
-// change speed only (results are identical for every choice), so a context
-// whose device, grids, field devices and fixed launch options match an
-// earlier one reuses that tuning instead of timing ~30 launches again.
-struct TuneKey {
-    int device, kind;                 // kind 0: dose path, 1: influence matrices
-    int ct[3], sg[3];
-    unsigned long long fields;        // per set beam: range shifter, aperture, divergent walls, vertex count
-    int block, aggregate, chunk;      // launch options the caller fixed
-    bool operator==(const TuneKey& o) const
-    {
-        return device == o.device && kind == o.kind && ct[0] == o.ct[0] && ct[1] == o.ct[1] && ct[2] == o.ct[2] &&
-               sg[0] == o.sg[0] && sg[1] == o.sg[1] && sg[2] == o.sg[2] && fields == o.fields &&
-               block == o.block && aggregate == o.aggregate && chunk == o.chunk;
-    }
-};
-
-std::mutex g_tune_mu;
-std::vector<std::pair<TuneKey, TuneResult>> g_tune_cache;
-
-TuneKey tune_key(const vpmc_ctx* c, int kind, const vpmc_opts& o)
-{
-    TuneKey k{};
-    k.device = c->device;
-    k.kind = kind;
-    for (int i = 0; i < 3; ++i) {
-        k.ct[i] = c->ctg.n[i];
-        k.sg[i] = c->sg.n[i];
-    }
-    unsigned long long h = 1469598103934665603ull;             // FNV-1a over the fields' device kinds
-    for (int b = 0; b < kMaxBeams; ++b) {
-        const unsigned long long v = !c->beam_set[b] ? 0ull
-                                     : 1ull | (unsigned long long)c->beams[b].rs << 1 |
-                                           (unsigned long long)c->beams[b].ap << 2 |
-                                           (unsigned long long)(c->beams[b].ap_sad > 0.0f) << 3 |
-                                           (unsigned long long)c->beams[b].nvert << 4;
-        h = (h ^ v) * 1099511628211ull;
-    }
-    k.fields = h;
-    k.block = o.block_size;
-    k.aggregate = o.aggregate;
-    k.chunk = o.chunk;
-    return k;
-}
-
-bool tune_cache_get(const TuneKey& k, TuneResult* out)
-{
-    std::lock_guard<std::mutex> lock(g_tune_mu);
-    for (const auto& e : g_tune_cache)
-        if (e.first == k) {
-            *out = e.second;
-            return true;
-        }
-    return false;
-}
-
-void tune_cache_put(const TuneKey& k, const TuneResult& t)
-{
-    std::lock_guard<std::mutex> lock(g_tune_mu);
-    for (auto& e : g_tune_cache)
-        if (e.first == k) {
-            e.second = t;
-            return;
-        }
-    g_tune_cache.emplace_back(k, t);
-}
-
-TuneResult resolve_launch(const vpmc_opts& o, const TuneResult& t)
-{
-    TuneResult r = t;
-    if (o.block_size) r.block = o.block_size;
-    if (o.aggregate >= 0) r.aggregate = o.aggregate;
-    if (o.chunk) r.chunk = o.chunk;
-    if (!t.valid) r.dev_block = 512;
-    return r;
 }
 
 // Device time of the beam-line kernels and of the patient kernel over the
@@ -866,7 +715,6 @@ vpmc_status vpmc_set_aperture(vpmc_ctx* c, int beam_id, const vpmc_beam* b)
         c->beam_set[beam_id] = prev_set;
         return st;
     }
-    c->tune_dose.valid = c->tune_im.valid = false;
     return VPMC_OK;
 }
 
@@ -899,10 +747,12 @@ vpmc_status vpmc_run_spots(vpmc_ctx* c, const vpmc_spot* spots, int n_spots, con
     std::vector<DevItem> items;
     long long total = 0;
     double qmax = 0.0, e_in = 0.0;
+    bool unit_weight = true;
     const double fs = std::ldexp(1.0, o.frac_bits);
     for (int i = 0; i < n_spots; ++i) {
         const vpmc_spot& s = spots[i];
         if (s.n_hist == 0) continue;
+        unit_weight = unit_weight && s.weight == 1.0;
         DevItem it{};
         it.hist_off = total;
         it.E0 = (float)s.energy_mev;
@@ -946,19 +796,10 @@ vpmc_status vpmc_run_spots(vpmc_ctx* c, const vpmc_spot* spots, int n_spots, con
         p.n_scen = 1;
         p.total = total;
         p.scratch = c->d_acc;
+        p.unit_weight = unit_weight ? 1 : 0;
         st = ensure_phase(c, total, p.surrogate != 0);
         if (st != VPMC_OK) return st;
-        const bool want_tune = o.block_size == 0 || o.aggregate < 0 || o.chunk == 0;
-        if (want_tune && !c->tune_dose.valid) {
-            const TuneKey key = tune_key(c, 0, o);
-            if (!tune_cache_get(key, &c->tune_dose)) {
-                st = autotune(c, p, &c->tune_dose, o);
-                if (st != VPMC_OK) return st;
-                CUDA_TRY(cudaMemsetAsync(c->d_acc, 0, c->nvox * sizeof(unsigned long long), c->stream));
-                tune_cache_put(key, c->tune_dose);
-            }
-        }
-        const TuneResult t = resolve_launch(o, c->tune_dose);
+        const LaunchShape t = launch_shape(o);
         st = reset_counters(c);
         if (st != VPMC_OK) return st;
         CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
@@ -1412,18 +1253,7 @@ vpmc_status vpmc_influence_matrix(vpmc_ctx* c, const vpmc_spot* spots, int n_spo
         p.records = nullptr;
         p.rec_cap = 0;
         p.ovf_count = d_ovf_count;
-        const bool want_tune = o.block_size == 0 || o.aggregate < 0 || o.chunk == 0;
-        if (want_tune && !c->tune_im.valid) {
-            const TuneKey key = tune_key(c, 1, o);
-            if (!tune_cache_get(key, &c->tune_im)) {
-                p.ovf = c->d_ovf;
-                p.ovf_cap = c->ovf_cap;
-                IM_TRY(cudaMemsetAsync(d_ovf_count, 0, sizeof(unsigned long long), c->stream));
-                IM_ST(autotune(c, p, &c->tune_im, o));
-                tune_cache_put(key, c->tune_im);
-            }
-        }
-        const TuneResult tr = resolve_launch(o, c->tune_im);
+        const LaunchShape tr = launch_shape(o);
         unsigned long long n_ovf = 0;
         for (int attempt = 0;; ++attempt) {
             p.ovf = c->d_ovf;
@@ -1948,7 +1778,7 @@ vpmc_status vpmc_surrogate_tracks(vpmc_ctx* c, const int* beam_ids, int n_beams,
     if (st != VPMC_OK) return done(st);
     if (use_surrogate && cudaMemsetAsync(c->sur.status, 0, sizeof(int), c->stream) != cudaSuccess)
         return done(fail(VPMC_ERR_CUDA, "status reset failed"));
-    const int block = c->tune_dose.valid ? c->tune_dose.dev_block : 512;
+    const int block = launch_shape(o).dev_block;
     for (long long h0 = 0; h0 < total; h0 += batch) {
         p.hist_begin = h0;
         p.total = std::min(total, h0 + batch);

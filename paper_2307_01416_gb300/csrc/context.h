@@ -10,14 +10,29 @@
 
 namespace vpmc {
 
-// Launch configuration of the two transport kernels chosen by the autotuner.
-struct TuneResult {
-    bool valid = false;
-    int dev_block = 512;     // k_devices threads per block
-    int block = 640;         // k_patient threads per block
+// Launch configuration of the transport kernels: the caller's options, else
+// one shape for every call, a full block per SM and chunks of one warp.  With
+// a deposit per voxel visit (patient.cu) it is the fastest of blocks of 512
+// to 896 threads, plain or warp-aggregated atomics and chunks of 16 to 128 on
+// every workload measured, or within 1 % of it (3.2e7 histories in the head:
+// 134 ms at 896 threads, 135 at 768, 162 at 512; aggregated atomics 227 ms;
+// chunks of 128 134.6 ms there and 4.6 against 4.1 ms on 4e6 histories behind
+// an aperture), so nothing is timed before a context's first call.
+struct LaunchShape {
+    int dev_block = 640;     // k_aperture threads per block (a full block; 512: 8 % slower behind an aperture)
+    int block = 896;         // k_patient threads per block
     int aggregate = 0;
     int chunk = 32;
 };
+
+inline LaunchShape launch_shape(const vpmc_opts& o)
+{
+    LaunchShape r;
+    if (o.block_size) r.block = o.block_size;
+    if (o.aggregate >= 0) r.aggregate = o.aggregate;
+    if (o.chunk) r.chunk = o.chunk;
+    return r;
+}
 
 // Grow-only device buffer a context keeps between calls (the influence
 // matrix's work arrays), so that repeated calls of one size allocate nothing.
@@ -84,7 +99,6 @@ struct vpmc_ctx {
     vpmc::SurQuery* d_sq = nullptr;            // brass entries handed to the surrogate
     long long sq_cap = 0;
     unsigned long long* d_sq_count = nullptr;
-    vpmc::TuneResult tune_dose, tune_im;
     long long launches = 0;                    // kernels launched since creation
     // per transport batch: events before the beam-line kernels, between them
     // and the patient kernel, and after it (the first kTimedBatches batches)

@@ -166,6 +166,7 @@ extern "C" vpmc_status vpmc_run_spots_noalloc(vpmc_ctx* c, const vpmc_spot* spot
     int n_items = 0, in_chunk = 0;
     long long total = 0;
     double qmax = 0.0, e_in = 0.0;
+    bool unit_weight = true;
     for (int i = 0; i < n_spots; ++i) {
         const vpmc_spot& s = spots[i];
         if (s.beam < 0 || s.beam >= kMaxBeams || !c->beam_set[s.beam])
@@ -178,6 +179,7 @@ extern "C" vpmc_status vpmc_run_spots_noalloc(vpmc_ctx* c, const vpmc_spot* spot
             !(s.weight >= 0.0))
             return report_error(VPMC_ERR_ARG, "spot %d: invalid position, sigma, divergence or weight", i);
         if (s.n_hist == 0) continue;
+        unit_weight = unit_weight && s.weight == 1.0;
         if (n_items == kMaxItems)
             return report_error(VPMC_ERR_ARG, "more than %d spots with histories; this entry point holds %d", kMaxItems,
                                 kMaxItems);
@@ -243,6 +245,7 @@ extern "C" vpmc_status vpmc_run_spots_noalloc(vpmc_ctx* c, const vpmc_spot* spot
     p.stats = counters + 3;
     p.status = status;
     p.scratch = acc;
+    p.unit_weight = unit_weight ? 1 : 0;
     p.phase = phase;
     p.phase_cap = kBatch;
     p.n_rep = 1;
@@ -260,20 +263,18 @@ extern "C" vpmc_status vpmc_run_spots_noalloc(vpmc_ctx* c, const vpmc_spot* spot
     p.max_iter = o.timeout_iters > 0 ? (int)o.timeout_iters : kMaxIter;
     p.records = reinterpret_cast<HistRecord*>(o.history_out);
     p.rec_cap = o.history_out ? o.history_cap : 0;
-    const TuneResult& t = c->tune_dose;
-    const int dev_block = t.valid ? t.dev_block : 512;
-    const int block = o.block_size ? o.block_size : (t.valid ? t.block : 640);
-    p.aggregate = o.aggregate >= 0 ? o.aggregate : (t.valid ? t.aggregate : 0);
-    p.chunk = o.chunk ? o.chunk : (t.valid ? t.chunk : 32);
+    const LaunchShape t = launch_shape(o);
+    p.aggregate = t.aggregate;
+    p.chunk = t.chunk;
     if (n_items) NA_TRY(cudaEventRecord(c->ev0, c->stream));
     for (long long h0 = 0; h0 < total; h0 += kBatch) {
         p.hist_begin = h0;
         p.total = h0 + kBatch < total ? h0 + kBatch : total;
         NA_TRY(cudaMemsetAsync(p.counter, 0, sizeof(unsigned long long), c->stream));
         NA_TRY(cudaMemsetAsync(p.phase_count, 0, sizeof(unsigned long long), c->stream));
-        NA_TRY(launch_devices(p, c->num_sms, dev_block, c->stream));
+        NA_TRY(launch_devices(p, c->num_sms, t.dev_block, c->stream));
         NA_TRY(cudaMemsetAsync(p.counter, 0, sizeof(unsigned long long), c->stream));
-        NA_TRY(launch_patient(p, c->num_sms, block, c->stream));
+        NA_TRY(launch_patient(p, c->num_sms, t.block, c->stream));
         c->launches += 3;
     }
     if (n_items) NA_TRY(cudaEventRecord(c->ev1, c->stream));

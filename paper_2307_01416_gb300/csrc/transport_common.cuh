@@ -144,6 +144,7 @@ struct Lane {
 
 // State of the history a patient lane carries.  Its global index and work
 // item stay in shared memory: they are read only when the history ends.
+template <class DepT>
 struct PatientLane {
     float p[3], d[3];
     float E, R, nlam;
@@ -151,7 +152,8 @@ struct PatientLane {
     uint32_t hist;              // history index within its spot
     int iters;
     int ic[3], is[3];
-    unsigned long long hdep;    // fixed-point energy the history deposited in the patient
+    DepT hdep;                  // fixed-point energy the history deposited in the patient
+    DepT pend;                  // influence-matrix mode: hdep at the last scoring; else the weighted deposits not yet scored
 };
 
 // kAllPhysics: scattering, straggling and nuclear removal all on, known at
