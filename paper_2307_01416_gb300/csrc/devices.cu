@@ -232,6 +232,7 @@ __global__ void __launch_bounds__(768, 1) k_source_rs(const TransportParams P)
     for (int k = 0; k < 3; ++k) { L.p[k] = 0.0f; L.d[k] = 0.0f; }
     unsigned long long acc_leak = 0, acc_rs = 0, acc_nuc = 0, acc_steps = 0, acc_err = 0;
     uint2 key = make_uint2(0u, 0u);
+    auto draw = [&](uint32_t step) { return philox(make_uint4(L.hist, step, 1u, 0u), key); };
 
     for (;;) {
         // ---- new histories for lanes whose history has ended ----
@@ -319,7 +320,7 @@ __global__ void __launch_bounds__(768, 1) k_source_rs(const TransportParams P)
                 else if (L.d[2] < 0.0f) { s_geom = __fdividef(B.rs_tup - L.p[2], L.d[2]); down = false; }
                 s_geom = fmaxf(s_geom, 0.0f);       // scattering offsets can leave it past the plane
                 StepResult o;
-                ch_step<kAllPhysics>(pmma, s_geom, L, P, key, o);
+                ch_step<kAllPhysics>(pmma, s_geom, L, P, draw, o);
                 acc_steps += 1;
                 const unsigned long long qs = to_fixed(o.dE, P.fscale, P.fx32);
                 acc_rs += qs;
@@ -431,6 +432,7 @@ __global__ void __launch_bounds__(640, 1) k_aperture(const TransportParams P)
     for (int k = 0; k < 3; ++k) { L.p[k] = 0.0f; L.d[k] = 0.0f; }
     unsigned long long acc_leak = 0, acc_ap = 0, acc_nuc = 0, acc_steps = 0, acc_err = 0;
     uint2 key = make_uint2(0u, 0u);
+    auto draw = [&](uint32_t step) { return philox(make_uint4(L.hist, step, 1u, 0u), key); };
 
     for (;;) {
         // ---- new histories for lanes whose history has ended ----
@@ -719,7 +721,7 @@ __global__ void __launch_bounds__(640, 1) k_aperture(const TransportParams P)
             }
             if (do_ch) {
                 StepResult o;
-                ch_step<kAllPhysics>(m, s_geom, L, P, key, o);
+                ch_step<kAllPhysics>(m, s_geom, L, P, draw, o);
                 acc_steps += 1;
                 const unsigned long long qs = to_fixed(o.dE, P.fscale, P.fx32);
                 acc_ap += qs;

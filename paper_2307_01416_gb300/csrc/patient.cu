@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(kPatientMaxBlock, 1) k_patient(const Transport
     long long* s_g = reinterpret_cast<long long*>(smem + PatientSmem::G);
     long long* s_pool = reinterpret_cast<long long*>(smem + PatientSmem::Pool) + 2 * warp;
     int* s_item = reinterpret_cast<int*>(smem + PatientSmem::Item);
+    uint4* s_rng = reinterpret_cast<uint4*>(smem + PatientSmem::Rng);
     {
         float2* R = reinterpret_cast<float2*>(smem + PatientSmem::R);
         float2* Et = reinterpret_cast<float2*>(smem + PatientSmem::Einv);
@@ -83,7 +84,7 @@ __global__ void __launch_bounds__(kPatientMaxBlock, 1) k_patient(const Transport
 
     bool alive = false, done = false;
     PatientLane<DepT> L;
-    L.hist = 0; L.hdep = 0; L.pend = 0; L.iters = 0; L.step = 0; L.E = 0.0f; L.R = 0.0f; L.nlam = 0.0f;
+    L.hdep = 0; L.pend = 0; L.iters = 0; L.step = 0; L.E = 0.0f; L.R = 0.0f; L.nlam = 0.0f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) { L.p[k] = 0.0f; L.d[k] = 0.0f; L.ic[k] = 0; L.is[k] = 0; }
     uint32_t key1 = 0u;
@@ -92,6 +93,8 @@ __global__ void __launch_bounds__(kPatientMaxBlock, 1) k_patient(const Transport
     unsigned long long* box_q = nullptr;
     bx.base = 0; bx.lo[0] = bx.lo[1] = bx.lo[2] = 0; bx.n[0] = bx.n[1] = bx.n[2] = 0;
     float wsc = 0.0f;
+
+    auto draw = [&](uint32_t step) { return philox_step(step, make_uint2(P.key0, key1), s_rng[threadIdx.x]); };
 
     for (;;) {
         // ---- histories handed over by the devices kernel ----
@@ -123,7 +126,6 @@ __global__ void __launch_bounds__(kPatientMaxBlock, 1) k_patient(const Transport
                         const DevItem I = P.items[r.item];
                         s_item[threadIdx.x] = r.item;
                         s_g[threadIdx.x] = r.g;
-                        L.hist = (uint32_t)(r.g - I.hist_off);
                         L.step = r.step;
                         L.iters = 0;
                         L.E = r.E;
@@ -131,6 +133,7 @@ __global__ void __launch_bounds__(kPatientMaxBlock, 1) k_patient(const Transport
                         L.hdep = 0;
                         L.pend = 0;
                         key1 = P.key1_hi ^ (uint32_t)I.spot;
+                        s_rng[threadIdx.x] = philox_step_prepare((uint32_t)(r.g - I.hist_off), make_uint2(P.key0, key1));
                         spr_scale = scens[I.scen].spr_scale;
                         bx = P.boxes[I.box];
                         box_q = P.scratch + bx.base;
@@ -241,7 +244,7 @@ __global__ void __launch_bounds__(kPatientMaxBlock, 1) k_patient(const Transport
                     s_geom = fminf(s_geom, nested ? dc[k] : fminf(dc[k], ds[k]));
                     d_old[k] = Dk;
                 }
-                ch_step<(kMode & kModeAllPhysics) != 0>(water, s_geom, L, P, make_uint2(P.key0, key1), o);
+                ch_step<(kMode & kModeAllPhysics) != 0>(water, s_geom, L, P, draw, o);
                 const unsigned long long qs = to_fixed(o.dE, P.fscale, kIM || P.fx32);
                 L.hdep += (DepT)qs;
                 if (!kIM) {

@@ -149,7 +149,6 @@ struct PatientLane {
     float p[3], d[3];
     float E, R, nlam;
     uint32_t step;              // condensed-history steps so far (RNG counter)
-    uint32_t hist;              // history index within its spot
     int iters;
     int ic[3], is[3];
     DepT hdep;                  // fixed-point energy the history deposited in the patient
@@ -159,8 +158,10 @@ struct PatientLane {
 // kAllPhysics: scattering, straggling and nuclear removal all on, known at
 // compile time, so that the step carries none of their switches; otherwise
 // the launch's switches decide.
-template <bool kAllPhysics, class LaneT>
-__device__ __forceinline__ void ch_step(const Medium& m, float s_geom, LaneT& L, const TransportParams& P, uint2 key,
+// draw(step): the step's random block, philox((history, step, 1, 0)) of the
+// history's key.
+template <bool kAllPhysics, class LaneT, class Draw>
+__device__ __forceinline__ void ch_step(const Medium& m, float s_geom, LaneT& L, const TransportParams& P, Draw&& draw,
                                         StepResult& o)
 {
     const bool mcs = kAllPhysics || P.mcs, straggling = kAllPhysics || P.straggling,
@@ -186,8 +187,8 @@ __device__ __forceinline__ void ch_step(const Medium& m, float s_geom, LaneT& L,
     // random numbers of this step: one block, counter (history, step, 1, 0),
     // six 21-bit uniforms -- the top 21 bits of each word (scattering) and the
     // low bits of words 0|1 and 2|3 (straggling)
-    uint4 r = make_uint4(L.hist, L.step, 1u, 0u);
-    if (mcs || straggling) r = philox(r, key);
+    uint4 r = make_uint4(0u, 0u, 0u, 0u);
+    if (mcs || straggling) r = draw(L.step);
 
     const float R1 = R0 - s * m.kappa;
     // (looked up whatever the sign of R1, the index being clamped, so that the

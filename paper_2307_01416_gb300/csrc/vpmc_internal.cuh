@@ -255,7 +255,9 @@ struct PatientSmem {                 // voxelised patient
     static constexpr size_t G = (Scens + sizeof(DevScen) * kMaxScen + 15) & ~size_t(15);
     static constexpr size_t Pool = G + sizeof(long long) * kPatientMaxBlock;
     static constexpr size_t Item = Pool + 2 * sizeof(long long) * (kPatientMaxBlock / 32);
-    static constexpr size_t Bytes = Item + sizeof(int) * kPatientMaxBlock;
+    // per thread: the words of its history's step blocks that do not depend on the step
+    static constexpr size_t Rng = (Item + sizeof(int) * kPatientMaxBlock + 15) & ~size_t(15);
+    static constexpr size_t Bytes = Rng + sizeof(uint4) * kPatientMaxBlock;
 };
 // One block per SM of each transport kernel: every layout fits the 227 KB a
 // block may opt in to.
