@@ -169,6 +169,8 @@ vpmc_status upload_beams(vpmc_ctx* c)
     std::vector<float> kappa;
     std::vector<unsigned char> ras;
     std::vector<float> ras_lb;
+    std::vector<uint16_t> near;
+    std::vector<uint32_t> local;
     DevBeam tmp[kMaxBeams];
     for (int b = 0; b < kMaxBeams; ++b) {
         tmp[b] = c->beams[b];
@@ -180,8 +182,11 @@ vpmc_status upload_beams(vpmc_ctx* c)
         kappa.resize(poly.size());
         polygon_curvature(c->poly[b].data(), nv, kappa.data() + (poly.size() - nv));
         tmp[b].ras_off = (int)ras.size();
-        ras.insert(ras.end(), c->raster[b].begin(), c->raster[b].end());
-        ras_lb.insert(ras_lb.end(), c->raster_lb[b].begin(), c->raster_lb[b].end());
+        const Raster& r = c->raster[b];
+        ras.insert(ras.end(), r.cells.begin(), r.cells.end());
+        ras_lb.insert(ras_lb.end(), r.lower.begin(), r.lower.end());
+        near.insert(near.end(), r.near.begin(), r.near.end());
+        local.insert(local.end(), r.local.begin(), r.local.end());
     }
     if (poly.size() > (size_t)kMaxPolyVerts)
         return fail(VPMC_ERR_ARG, "aperture polygons have %zu vertices in total (max %d)", poly.size(), kMaxPolyVerts);
@@ -189,6 +194,10 @@ vpmc_status upload_beams(vpmc_ctx* c)
     cudaFree(c->d_poly_kappa);
     cudaFree(c->d_raster);
     cudaFree(c->d_raster_lb);
+    cudaFree(c->d_raster_near);
+    cudaFree(c->d_raster_local);
+    c->d_raster_near = nullptr;
+    c->d_raster_local = nullptr;
     c->d_poly = nullptr;
     c->d_poly_kappa = nullptr;
     c->d_raster = nullptr;
@@ -199,6 +208,12 @@ vpmc_status upload_beams(vpmc_ctx* c)
         CUDA_TRY(cudaMemcpy(c->d_poly_kappa, kappa.data(), kappa.size() * sizeof(float), cudaMemcpyHostToDevice));
     CUDA_TRY(dev_alloc(&c->d_raster, std::max<size_t>(ras.size(), 1)));
     CUDA_TRY(dev_alloc(&c->d_raster_lb, std::max<size_t>(ras_lb.size(), 1)));
+    CUDA_TRY(dev_alloc(&c->d_raster_near, std::max<size_t>(near.size(), 1)));
+    CUDA_TRY(dev_alloc(&c->d_raster_local, std::max<size_t>(local.size(), 1)));
+    if (!near.empty()) {
+        CUDA_TRY(cudaMemcpy(c->d_raster_near, near.data(), near.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
+        CUDA_TRY(cudaMemcpy(c->d_raster_local, local.data(), local.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
+    }
     if (!poly.empty()) CUDA_TRY(cudaMemcpy(c->d_poly, poly.data(), poly.size() * sizeof(float2), cudaMemcpyHostToDevice));
     if (!ras.empty()) CUDA_TRY(cudaMemcpy(c->d_raster, ras.data(), ras.size(), cudaMemcpyHostToDevice));
     if (!ras_lb.empty())
@@ -338,6 +353,8 @@ TransportParams base_params(vpmc_ctx* c, const vpmc_opts& o)
     p.n_poly = c->n_poly;
     p.raster = c->d_raster;
     p.raster_lb = c->d_raster_lb;
+    p.raster_near = c->d_raster_near;
+    p.raster_local = c->d_raster_local;
     p.range_rejection = o.range_rejection;
     p.items = c->d_items;
     p.boxes = c->d_boxes;
@@ -650,8 +667,7 @@ vpmc_status vpmc_set_aperture(vpmc_ctx* c, int beam_id, const vpmc_beam* b)
     }
     d.ap = b->ap_present ? 1 : 0;
     std::vector<double> poly;
-    std::vector<unsigned char> ras;
-    std::vector<float> ras_lb;
+    Raster ras{};
     if (d.ap) {
         if (!b->poly_xy || b->n_vertices < 3) return fail(VPMC_ERR_ARG, "aperture needs a polygon of >= 3 vertices");
         if (!(b->ap_thickness_mm > 0)) return fail(VPMC_ERR_ARG, "aperture thickness must be positive");
@@ -687,11 +703,10 @@ vpmc_status vpmc_set_aperture(vpmc_ctx* c, int beam_id, const vpmc_beam* b)
             d.ap_K = 1.0f;
             d.ap_cos = 1.0f;
         }
-        ras.resize(kRaster * kRaster);
-        ras_lb.resize(kRaster * kRaster);
         // range rejection needs wall distances up to half the block thickness only
-        build_raster(poly.data(), b->n_vertices, (0.5 * b->ap_thickness_mm + 1.0) * margin_scale, ras.data(),
-                     ras_lb.data(), d.ras_lo, d.ras_inv, &d.ras_diag);
+        build_raster(poly.data(), b->n_vertices, (0.5 * b->ap_thickness_mm + 1.0) * margin_scale, &ras);
+        for (int k = 0; k < 2; ++k) { d.ras_lo[k] = ras.lo[k]; d.ras_inv[k] = ras.inv[k]; }
+        d.ras_diag = ras.diag;
         d.nvert = b->n_vertices;
     }
     if (first_device < 1e300 && !(-b->source_to_iso_mm < first_device))
@@ -699,19 +714,16 @@ vpmc_status vpmc_set_aperture(vpmc_ctx* c, int beam_id, const vpmc_beam* b)
     const bool prev_set = c->beam_set[beam_id];
     const DevBeam prev = c->beams[beam_id];
     std::vector<double> prev_poly = c->poly[beam_id];
-    std::vector<unsigned char> prev_ras = c->raster[beam_id];
-    std::vector<float> prev_lb = c->raster_lb[beam_id];
+    Raster prev_ras = c->raster[beam_id];
     c->beams[beam_id] = d;
     c->poly[beam_id] = poly;
     c->raster[beam_id] = ras;
-    c->raster_lb[beam_id] = ras_lb;
     c->beam_set[beam_id] = true;
     vpmc_status st = upload_beams(c);
     if (st != VPMC_OK) {
         c->beams[beam_id] = prev;
         c->poly[beam_id] = prev_poly;
         c->raster[beam_id] = prev_ras;
-        c->raster_lb[beam_id] = prev_lb;
         c->beam_set[beam_id] = prev_set;
         return st;
     }
@@ -1477,6 +1489,8 @@ void vpmc_destroy(vpmc_ctx* c)
     cudaFree(c->d_poly);
     cudaFree(c->d_raster);
     cudaFree(c->d_raster_lb);
+    cudaFree(c->d_raster_near);
+    cudaFree(c->d_raster_local);
     cudaFree(c->d_counter);
     cudaFree(c->d_stats);
     cudaFree(c->d_status);

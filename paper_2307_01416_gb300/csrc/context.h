@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "../../include/vpmc.h"
+#include "tables.h"
 #include "vpmc_internal.cuh"
 
 namespace vpmc {
@@ -19,7 +20,7 @@ namespace vpmc {
 // chunks of 128 134.6 ms there and 4.6 against 4.1 ms on 4e6 histories behind
 // an aperture), so nothing is timed before a context's first call.
 struct LaunchShape {
-    int dev_block = 640;     // k_aperture threads per block (a full block; 512: 8 % slower behind an aperture)
+    int dev_block = 768;     // k_aperture threads per block (a full block)
     int block = 896;         // k_patient threads per block
     int aggregate = 0;
     int chunk = 32;
@@ -66,13 +67,14 @@ struct vpmc_ctx {
     bool beam_set[vpmc::kMaxBeams]{};
     vpmc::DevBeam beams[vpmc::kMaxBeams]{};
     std::vector<double> poly[vpmc::kMaxBeams];
-    std::vector<unsigned char> raster[vpmc::kMaxBeams];
-    std::vector<float> raster_lb[vpmc::kMaxBeams];
+    vpmc::Raster raster[vpmc::kMaxBeams];
     vpmc::DevBeam* d_beams = nullptr;
     float2* d_poly = nullptr;
     int n_poly = 0;
     unsigned char* d_raster = nullptr;
     float* d_raster_lb = nullptr;
+    uint16_t* d_raster_near = nullptr;
+    uint32_t* d_raster_local = nullptr;
     // per-launch buffers
     unsigned long long* d_counter = nullptr;
     unsigned long long* d_stats = nullptr;

@@ -150,6 +150,55 @@ bool crossing_number_inside(const double* xy, int n, double x, double y)
     return inside;
 }
 
+// Crossing-number test of the points of a cell [x0, x1] x [y0, y1] (grown by
+// the FP32 placement margin): the edges (i - 1, i) that it has to evaluate as
+// a cyclic run, first | count << 16, and in bit 31 the parity of the rest.
+// Edges that miss the cell's height or lie left of it never count.  Edges
+// right of it count when they straddle the point's height; their number has
+// one parity over the whole cell when every vertex of theirs within its
+// height joins two of them, so an edge that meets an evaluated one there is
+// evaluated too.  0: no run of at most kLocalMax edges holds them.
+uint32_t local_edges(const double* xy, int n, double x0, double y0, double x1, double y1,
+                     std::vector<unsigned char>& kind)
+{
+    auto X = [&](int i) { return xy[2 * ((i + n) % n)]; };
+    auto Y = [&](int i) { return xy[2 * ((i + n) % n) + 1]; };
+    enum { kOut = 0, kEval = 1, kRight = 2 };
+    for (int i = 0; i < n; ++i) {
+        const double xa = X(i - 1), ya = Y(i - 1), xb = X(i), yb = Y(i);
+        if (std::max(ya, yb) < y0 || std::min(ya, yb) > y1 || std::max(xa, xb) < x0) kind[i] = kOut;
+        else kind[i] = std::min(xa, xb) > x1 ? kRight : kEval;
+    }
+    // edge i ends in vertex i, edge i + 1 starts there
+    for (bool grew = true; grew;) {
+        grew = false;
+        for (int i = 0; i < n; ++i) {
+            const int j = (i + 1) % n;
+            if (Y(i) < y0 || Y(i) > y1 || (kind[i] != kRight && kind[j] != kRight) || kind[i] == kind[j]) continue;
+            kind[kind[i] == kRight ? i : j] = kEval;
+            grew = true;
+        }
+    }
+    int first = -1, last = -1, gap = 0, start = 0;
+    for (int i = 0; i < n; ++i) {
+        if (kind[i] != kEval) continue;
+        if (first < 0) first = start = i;
+        else if (i - last > gap) { gap = i - last; start = i; }
+        last = i;
+    }
+    if (first < 0) return 0u;
+    if (first + n - last >= gap) { gap = first + n - last; start = first; }
+    const int count = n - gap + 1;
+    if (count > kLocalMax) return 0u;
+    int right = 0;                                   // of the edges outside the run
+    const double ym = 0.5 * (y0 + y1);
+    for (int k = count; k < n; ++k) {
+        const int i = (start + k) % n;
+        if (kind[i] == kRight) right += (Y(i - 1) > ym) != (Y(i) > ym);
+    }
+    return (uint32_t)start | (uint32_t)count << 16 | (uint32_t)(right & 1) << 31;
+}
+
 }  // namespace
 
 double pmma_stopping_power_ratio(double kinetic)
@@ -189,9 +238,15 @@ void build_tables(const double* curve15, TablesImage* img)
     }
 }
 
-void build_raster(const double* xy, int n, double margin, unsigned char* cells, float* lower, float lo[2], float inv[2],
-                  float* diag)
+void build_raster(const double* xy, int n, double margin, Raster* out)
 {
+    std::vector<unsigned char>& cells = out->cells;
+    std::vector<float>& lower = out->lower;
+    std::vector<uint16_t>& near = out->near;
+    cells.assign((size_t)kRaster * kRaster, 0);
+    lower.assign((size_t)kRaster * kRaster, 0.0f);
+    near.assign((size_t)kRaster * kRaster, 0);
+    out->local.assign((size_t)kRaster * kRaster, 0u);
     double xmin = xy[0], xmax = xy[0], ymin = xy[1], ymax = xy[1];
     for (int i = 1; i < n; ++i) {
         xmin = std::min(xmin, xy[2 * i]); xmax = std::max(xmax, xy[2 * i]);
@@ -202,39 +257,56 @@ void build_raster(const double* xy, int n, double margin, unsigned char* cells, 
     const double pad = std::max(0.02 * std::max(xmax - xmin, ymax - ymin) + 0.1, margin);
     xmin -= pad; xmax += pad; ymin -= pad; ymax += pad;
     const double cw = (xmax - xmin) / kRaster, ch = (ymax - ymin) / kRaster;
-    lo[0] = (float)xmin; lo[1] = (float)ymin;
-    inv[0] = (float)(1.0 / cw); inv[1] = (float)(1.0 / ch);
-    *diag = (float)(std::sqrt(cw * cw + ch * ch) * (1.0 + 1e-6) + 1e-4);
+    out->lo[0] = (float)xmin; out->lo[1] = (float)ymin;
+    out->inv[0] = (float)(1.0 / cw); out->inv[1] = (float)(1.0 / ch);
+    out->diag = (float)(std::sqrt(cw * cw + ch * ch) * (1.0 + 1e-6) + 1e-4);
     // FP32 placement of a point can move it by a few ulps across a cell border,
     // so a cell is classified only if no edge comes within eps of it
     const double eps = 1e-3 * std::max(cw, ch) + 1e-4 * (std::fabs(xmin) + std::fabs(ymin) + 1.0);
+    const double half = 0.5 * std::sqrt(cw * cw + ch * ch);
     // rows are independent: split them over the host's threads
     auto rows = [&](int cy_begin, int cy_end) {
+    std::vector<double> dist(n);                     // edge to the cell's centre
+    std::vector<unsigned char> kind(n);
     for (int cy = cy_begin; cy < cy_end; ++cy)
         for (int cx = 0; cx < kRaster; ++cx) {
             const double x0 = xmin + cx * cw - eps, x1 = xmin + (cx + 1) * cw + eps;
             const double y0 = ymin + cy * ch - eps, y1 = ymin + (cy + 1) * ch + eps;
+            const double mx = xmin + (cx + 0.5) * cw, my = ymin + (cy + 0.5) * ch;
+            double dmin = 1e300;
+            int nearest = 0;
+            for (int i = 0; i < n; ++i) {
+                const int j = i + 1 < n ? i + 1 : 0;
+                dist[i] = point_segment_distance(mx, my, xy[2 * i], xy[2 * i + 1], xy[2 * j], xy[2 * j + 1]);
+                if (dist[i] < dmin) { dmin = dist[i]; nearest = i; }
+            }
             bool edge = false;
             for (int i = 0; i < n && !edge; ++i) {
-                const int j = (i + 1) % n;
+                if (dist[i] > half + 2.0 * eps) continue;      // cannot reach the cell
+                const int j = i + 1 < n ? i + 1 : 0;
                 edge = segment_hits_box(xy[2 * i], xy[2 * i + 1], xy[2 * j], xy[2 * j + 1], x0, y0, x1, y1);
             }
             unsigned char c = 2;
-            if (!edge) c = crossing_number_inside(xy, n, xmin + (cx + 0.5) * cw, ymin + (cy + 0.5) * ch) ? 1 : 0;
+            if (!edge) c = crossing_number_inside(xy, n, mx, my) ? 1 : 0;
             cells[cy * kRaster + cx] = c;
-            // lower bound of the distance from any point of the cell to the boundary
+            // lower bound of the distance from any point of the cell to the
+            // boundary (an edge farther than dmin + half from the centre is
+            // farther from the cell than the nearest one)
             double lb = 0.0;
             if (!edge) {
                 lb = 1e300;
                 const double rx0 = xmin + cx * cw, rx1 = rx0 + cw, ry0 = ymin + cy * ch, ry1 = ry0 + ch;
                 for (int i = 0; i < n; ++i) {
-                    const int j = (i + 1) % n;
+                    if (dist[i] > dmin + half + 1e-9) continue;
+                    const int j = i + 1 < n ? i + 1 : 0;
                     lb = std::min(lb, segment_rect_distance(xy[2 * i], xy[2 * i + 1], xy[2 * j], xy[2 * j + 1],
                                                             rx0, ry0, rx1, ry1));
                 }
                 lb = std::max(lb - 1e-4, 0.0);     // margin for the FP32 use of the bound
             }
             lower[cy * kRaster + cx] = (float)lb;
+            near[cy * kRaster + cx] = (uint16_t)nearest;
+            if (edge) out->local[cy * kRaster + cx] = local_edges(xy, n, x0, y0, x1, y1, kind);
         }
     };
     const int nt = (int)std::max(1u, std::min(std::thread::hardware_concurrency(), 32u));

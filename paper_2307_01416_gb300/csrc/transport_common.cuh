@@ -131,8 +131,7 @@ struct Lane {
     float p[3], d[3];
     float E, R, nlam;
     uint32_t step;  // condensed-history steps so far (RNG counter)
-    uint32_t hist;  // history index within its spot
-    int stage;      // devices: -1 just born, 0 range shifter, 1 aperture
+    int stage;      // aperture: -1 just born, 1 in the block
     int forced;     // aperture: 1 the next step is in brass (after a wall hit), -1 on the entrance plane
     int ic[3], is[3];
     int item;

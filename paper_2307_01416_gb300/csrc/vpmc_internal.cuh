@@ -17,6 +17,7 @@ constexpr int kMaxBeams = 64;            // beam entries: fields, or (field, ene
 constexpr int kMaxScen = 64;
 constexpr int kMaxPolyVerts = 4096;
 constexpr int kRaster = 256;         // BEV raster per beam (cells per side): opening class, wall-distance bound
+constexpr int kLocalMax = 12;        // edges of a raster cell's crossing-number test
 constexpr float kEcut = 0.5f;        // MeV
 constexpr int kMaxIter = 200000;     // default cap on a history's iterations in one kernel (then it is an error)
 
@@ -49,7 +50,7 @@ struct DevBeam {
     float ap_tup, ap_tdn;
     int poly_off, nvert;
     float ras_lo[2], ras_inv[2];     // raster origin and 1/cell size
-    int ras_off;                     // offset into the raster arrays (class bytes, distance bounds)
+    int ras_off;                     // offset into the raster arrays (class bytes, distance bounds, nearest and local edges)
     float ras_diag;                  // raster cell diagonal
     float r_circ;                    // largest vertex distance from the beam axis (training tracks)
     float ap_sad;                    // divergent walls: virtual source at t = -ap_sad (0: parallel walls)
@@ -173,6 +174,9 @@ struct TransportParams {
     int n_poly;
     const unsigned char* raster;
     const float* raster_lb;          // per raster cell: lower bound of the distance to the opening's boundary
+    const uint16_t* raster_near;     // per raster cell: the edge nearest to its centre
+    const uint32_t* raster_local;    // per raster cell near an edge: the edges (i - 1, i) of its crossing-number
+                                     // test, first | count << 16, the others' parity in bit 31 (0: all edges)
     int range_rejection;             // absorb brass protons that cannot leave the block
     const DevItem* items;
     int n_items;
