@@ -140,6 +140,44 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// (a, b) + (c, d), each sum rounded as the scalar add.
+__device__ __forceinline__ float2 add2(float a, float b, float c, float d)
+{
+    float2 r;
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 x, x, y;\n\t"
+        "mov.b64 {%0, %1}, x;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a), "f"(b), "f"(c), "f"(d));
+    return r;
+}
+
+// relu of two BF16 values (a NaN becomes 0, as in fmaxf(x, 0)).
+__device__ __forceinline__ uint32_t relu_bf16x2(uint32_t h)
+{
+    uint32_t r;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0u));
+    return r;
+}
+
+// Bulk copies of bytes (a multiple of 16, both addresses 16-byte aligned):
+// global to shared memory, arriving on mbar; shared to global memory.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(mbar), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 :: "r"(dst), "l"(src), "r"(bytes), "r"(mbar) : "memory");
+}
+
+__device__ __forceinline__ void bulk_store(void* dst, uint32_t src, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" :: "l"(dst), "r"(src), "r"(bytes)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
+// Until this thread's bulk stores have read their source / are complete.
+__device__ __forceinline__ void bulk_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 {
     __nv_bfloat162 h = __floats2bfloat162_rn(a, b);   // a in the low half (lower address)
@@ -200,21 +238,12 @@ __device__ __forceinline__ bool group_sync_and(int g, bool ok)
     return all != 0u;
 }
 
-// publish / complete for one warpgroup's tile pipeline.
+// publish for one warpgroup's tile pipeline.
 __device__ __forceinline__ void publish_group(int g)
 {
     fence_async_smem();
     tc_fence_before();
     group_sync(g);
-}
-
-__device__ __forceinline__ bool complete_group(int g, uint32_t mbar, uint32_t& phase)
-{
-    const bool ok = mbar_wait(mbar, phase);
-    phase ^= 1u;
-    const bool all = group_sync_and(g, ok);
-    tc_fence_after();
-    return all;
 }
 
 __device__ __forceinline__ void copy_to_smem(unsigned char* dst, const unsigned char* src, int bytes)
@@ -264,16 +293,19 @@ __device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16])
 }
 
 // relu(D + b) of 16 columns [c0, c0 + 16) of row r, rounded to BF16 into the
-// K-major [128 x 128] tile dst.
-__device__ __forceinline__ void relu_pack16(const uint32_t (&v)[16], const float* __restrict__ bias, int c0,
-                                            unsigned char* dst, int r)
+// K-major [128 x 128] tile dst (bias in shared memory).  Packed adds, the
+// rounding before the relu (which commutes with it): 1.5 operations and a
+// quarter of a bias load per value.
+__device__ __forceinline__ void relu_pack16(const uint32_t (&v)[16], const float* bias, int c0, unsigned char* dst, int r)
 {
     uint32_t w[8];
 #pragma unroll
-    for (int j = 0; j < 16; j += 2) {
-        const float a0 = __uint_as_float(v[j]) + __ldg(bias + c0 + j);
-        const float a1 = __uint_as_float(v[j + 1]) + __ldg(bias + c0 + j + 1);
-        w[j >> 1] = pack_bf16(fmaxf(a0, 0.0f), fmaxf(a1, 0.0f));
+    for (int j = 0; j < 16; j += 4) {
+        const float4 b = *reinterpret_cast<const float4*>(bias + c0 + j);
+        const float2 p = add2(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), b.x, b.y);
+        const float2 q = add2(__uint_as_float(v[j + 2]), __uint_as_float(v[j + 3]), b.z, b.w);
+        w[j >> 1] = relu_bf16x2(pack_bf16(p.x, p.y));
+        w[(j >> 1) + 1] = relu_bf16x2(pack_bf16(q.x, q.y));
     }
     *reinterpret_cast<uint4*>(dst + kmaj(r, c0, kH)) = make_uint4(w[0], w[1], w[2], w[3]);
     *reinterpret_cast<uint4*>(dst + kmaj(r, c0 + 8, kH)) = make_uint4(w[4], w[5], w[6], w[7]);
@@ -302,8 +334,7 @@ __device__ __forceinline__ void tmem_cols_pipelined(uint32_t t_row, int ncols, F
 
 // Hidden-layer epilogue of the forward path: relu(D + b) to BF16 into the
 // K-major [128 x 128] tile dst.
-__device__ __forceinline__ void hidden_epilogue_fwd(uint32_t t_row, const float* __restrict__ bias,
-                                                    unsigned char* dst, int r)
+__device__ __forceinline__ void hidden_epilogue_fwd(uint32_t t_row, const float* bias, unsigned char* dst, int r)
 {
     tmem_cols_pipelined(t_row, kH, [&](const uint32_t (&v)[16], int c0) { relu_pack16(v, bias, c0, dst, r); });
 }
@@ -334,89 +365,117 @@ __device__ __forceinline__ void hidden_epilogue_train(uint32_t t_row, const floa
     });
 }
 
-// z = D3 + b3 for row r (48 columns, 45 used).
-__device__ __forceinline__ void output_epilogue(uint32_t t_d3, const float* __restrict__ b3, float (&z)[kOutPad])
+// z = D3 + b3 for row r (48 columns, 45 used; b3 in shared memory, padded with zeros).
+__device__ __forceinline__ void output_epilogue(uint32_t t_d3, const float* b3, float (&z)[kOutPad])
 {
     float v[32], u[16];
     tmem_ld32(t_d3, v);
     tmem_ld16(t_d3 + 32u, u);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) z[j] = v[j] + __ldg(b3 + j);
+    for (int j = 0; j < 32; ++j) z[j] = v[j] + b3[j];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) z[32 + j] = u[j] + (32 + j < kOut ? __ldg(b3 + 32 + j) : 0.0f);
+    for (int j = 0; j < 16; ++j) z[32 + j] = u[j] + b3[32 + j];
 }
 
 // ============================================================================
 // Forward: network outputs of n feature rows, and the same network drawing
 // exit states for the transport's queries.
 // ============================================================================
-// A CTA runs kGroups tile pipelines, one per 128-thread warpgroup, sharing
-// one copy of the weight images: while one group's epilogue runs on the CUDA
-// cores, another group's GEMMs run on the tensor core.  Per group: its input,
-// hidden and staging tiles, its queries and its mbarrier; in tensor memory,
-// 128 columns (D1, then D2 over it once D1 is read, then D3).
-constexpr int kGroups = 3;
-constexpr int kFwdThreads = kGroups * kRows;
+// A CTA runs kG tile pipelines, one per 128-thread warpgroup, sharing one copy
+// of the weight images and biases: while one group's epilogue runs on the CUDA
+// cores, another group's GEMMs run on the tensor core.  Per group: its input
+// and hidden tiles, its raw inputs (and queries) and its mbarriers; in tensor
+// memory, 128 columns (D1, then D2 over it once D1 is read, then D3).
+//
+// Forward: per 128 x 128 tile layer some 512 cycles of tensor core, 64 KB of
+// tensor-memory reads and 270 issue slots of epilogue per warp, so the three
+// are of one size (about 100 us each on 4.2e6 rows, whose 204 bytes a row
+// take 126 us of HBM) and the time is set by how well they overlap: four
+// groups, the next tile's inputs and the last one's outputs moved by bulk
+// copies, and one barrier per layer: 278 us (691 TFLOP/s).  520 us with three
+// groups, two barriers, scalar bias loads from global memory and copies
+// through registers.
+// Inference holds its queries in shared memory too: three groups fit.
+template <int kG, bool kQueries>
 struct FwdSmem {
     static constexpr int W = 0;                                   // W1, W2, W3 images
-    static constexpr int G0 = kImgW2T;                            // the groups' regions
+    static constexpr int Bias = kImgW2T;                          // b1, b2, b3 (padded), FP32
+    static constexpr int G0 = (Bias + (2 * kH + kOutPad) * 4 + 127) / 128 * 128;     // the groups' regions
     // offsets within a group's region
     static constexpr int X = 0;                                   // [128 x 16]
     static constexpr int H = X + kRows * kInPad * 2;              // [128 x 128]; also the output staging
     static constexpr int XS = H + kRows * kH * 2;                 // FP32 inputs of a tile, [128 x 6]
-    static constexpr int QS = XS + kRows * kIn * 4;               // a tile's queries (inference)
-    static constexpr int Bar = QS + kRows * (int)sizeof(SurQuery);
-    static constexpr int GBytes = (Bar + 8 + 127) / 128 * 128;
-    static constexpr int Slot = G0 + kGroups * GBytes;
+    static constexpr int QS = XS + (kQueries ? 0 : kRows * kIn * 4);    // a tile's queries (inference)
+    static constexpr int Bar = QS + (kQueries ? kRows * (int)sizeof(SurQuery) : 0);
+    static constexpr int GBytes = (Bar + 16 + 127) / 128 * 128;
+    static constexpr int Slot = G0 + kG * GBytes;
     static constexpr int Bytes = Slot + 8;
+    static_assert(G0 % 128 == 0 && GBytes % 128 == 0, "operand tiles 128-byte aligned");
+    static_assert(Bytes <= 232448, "the CTA exceeds the shared memory of one SM");
 };
-static_assert(FwdSmem::Bytes <= 232448, "forward CTA exceeds the shared memory of one SM");
-static_assert(FwdSmem::G0 % 128 == 0 && FwdSmem::GBytes % 128 == 0, "operand tiles 128-byte aligned");
+constexpr int kFwdGroups = 4, kInferGroups = 3;
+using FwdS = FwdSmem<kFwdGroups, false>;
+using InferS = FwdSmem<kInferGroups, true>;
 constexpr uint32_t kFwdCols = 512;        // allocation (a power of two); group g uses columns [128 g, 128 g + 128)
 
-// The three GEMMs of one tile whose inputs are in the group's X; returns
-// false when a tensor-core wait failed.  On return the group's accumulator
-// columns hold z - b3.
-__device__ __forceinline__ bool forward_tile(unsigned char* sm, unsigned char* gs, uint32_t tcol, uint32_t t_row,
-                                             const SurNet& net, uint32_t bar, uint32_t& phase, int r, int g)
+// The three GEMMs of one tile whose inputs are in the group's X and published;
+// clears ok when a tensor-core wait failed (the caller's group agrees on it).
+// On return the group's accumulator columns hold z - b3.
+template <class S>
+__device__ __forceinline__ void forward_tile(unsigned char* sm, unsigned char* gs, uint32_t tcol, uint32_t t_row,
+                                             uint32_t& phase, int r, int g, bool& ok)
 {
-    const uint32_t s0 = smem_addr(sm), gs0 = smem_addr(gs);
+    const uint32_t s0 = smem_addr(sm), gs0 = smem_addr(gs), bar = gs0 + S::Bar;
+    const float* bias = reinterpret_cast<const float*>(sm + S::Bias);
+    if (r == 0) {
+        tc_fence_after();
+        mma_tile(tcol, gs0 + S::X, s0 + S::W + kImgW1, kInPad, kH, false);
+        umma_commit(bar);
+    }
+    ok = mbar_wait(bar, phase) && ok;
+    phase ^= 1u;
+    tc_fence_after();
+    hidden_epilogue_fwd(t_row, bias, gs + S::H, r);
     publish_group(g);
     if (r == 0) {
         tc_fence_after();
-        mma_tile(tcol, gs0 + FwdSmem::X, s0 + FwdSmem::W + kImgW1, kInPad, kH, false);
+        mma_tile(tcol, gs0 + S::H, s0 + S::W + kImgW2, kH, kH, false);
         umma_commit(bar);
     }
-    if (!complete_group(g, bar, phase)) return false;
-    hidden_epilogue_fwd(t_row, net.params + ob1, gs + FwdSmem::H, r);
+    ok = mbar_wait(bar, phase) && ok;
+    phase ^= 1u;
+    tc_fence_after();
+    hidden_epilogue_fwd(t_row, bias + kH, gs + S::H, r);
     publish_group(g);
     if (r == 0) {
         tc_fence_after();
-        mma_tile(tcol, gs0 + FwdSmem::H, s0 + FwdSmem::W + kImgW2, kH, kH, false);
+        mma_tile(tcol, gs0 + S::H, s0 + S::W + kImgW3, kH, kOutPad, false);
         umma_commit(bar);
     }
-    if (!complete_group(g, bar, phase)) return false;
-    hidden_epilogue_fwd(t_row, net.params + ob2, gs + FwdSmem::H, r);
-    publish_group(g);
-    if (r == 0) {
-        tc_fence_after();
-        mma_tile(tcol, gs0 + FwdSmem::H, s0 + FwdSmem::W + kImgW3, kH, kOutPad, false);
-        umma_commit(bar);
-    }
-    return complete_group(g, bar, phase);
+    ok = mbar_wait(bar, phase) && ok;
+    phase ^= 1u;
+    tc_fence_after();
 }
 
+template <class S, int kG>
 __device__ __forceinline__ void fwd_prologue(unsigned char* sm, const SurNet& net, uint32_t& tbase)
 {
-    copy_to_smem(sm + FwdSmem::W, net.img, kImgW2T);
-    if (threadIdx.x < kGroups) mbar_init(smem_addr(sm + FwdSmem::G0 + threadIdx.x * FwdSmem::GBytes + FwdSmem::Bar));
-    if ((threadIdx.x >> 5) == 0) tmem_alloc(smem_addr(sm + FwdSmem::Slot), kFwdCols);
+    copy_to_smem(sm + S::W, net.img, kImgW2T);
+    float* bias = reinterpret_cast<float*>(sm + S::Bias);
+    for (int i = threadIdx.x; i < 2 * kH + kOutPad; i += blockDim.x)
+        bias[i] = i < kH ? net.params[ob1 + i]
+                         : (i < 2 * kH ? net.params[ob2 + i - kH] : (i < 2 * kH + kOut ? net.params[ob3 + i - 2 * kH] : 0.0f));
+    if (threadIdx.x < 2 * kG)
+        mbar_init(smem_addr(sm + S::G0 + (threadIdx.x >> 1) * S::GBytes + S::Bar + 8 * (threadIdx.x & 1)));
+    fence_async_smem();
+    if ((threadIdx.x >> 5) == 0) tmem_alloc(smem_addr(sm + S::Slot), kFwdCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    tbase = *reinterpret_cast<volatile uint32_t*>(sm + FwdSmem::Slot);
+    tbase = *reinterpret_cast<volatile uint32_t*>(sm + S::Slot);
 }
 
+template <class S>
 __device__ __forceinline__ void fwd_epilogue_free(unsigned char* sm, uint32_t tbase, uint32_t bar, uint32_t phase,
                                                   bool ok, const SurNet& net)
 {
@@ -435,56 +494,75 @@ __device__ __forceinline__ void fwd_epilogue_free(unsigned char* sm, uint32_t tb
     }
 }
 
-__global__ void __launch_bounds__(kFwdThreads, 1) k_sur_forward(const SurNet net, const float* __restrict__ x,
-                                                                 long long n, float* __restrict__ z)
+__global__ void __launch_bounds__(kFwdGroups * kRows, 1) k_sur_forward(const SurNet net, const float* __restrict__ x,
+                                                                       long long n, float* __restrict__ z)
 {
+    using S = FwdS;
     extern __shared__ __align__(1024) unsigned char sm[];
     uint32_t tbase;
-    fwd_prologue(sm, net, tbase);
+    fwd_prologue<S, kFwdGroups>(sm, net, tbase);
     const int g = threadIdx.x / kRows, r = threadIdx.x % kRows;
-    unsigned char* gs = sm + FwdSmem::G0 + g * FwdSmem::GBytes;
+    unsigned char* gs = sm + S::G0 + g * S::GBytes;
     const uint32_t tcol = tbase + (uint32_t)(g * kRows);
     const uint32_t t_row = tcol + ((uint32_t)((r >> 5) * 32) << 16);
-    const uint32_t bar = smem_addr(gs + FwdSmem::Bar);
-    uint32_t phase = 0u;
-    bool ok = true;
-    float* xs = reinterpret_cast<float*>(gs + FwdSmem::XS);
-    float* zs = reinterpret_cast<float*>(gs + FwdSmem::H);
-    for (long long tile = (long long)blockIdx.x * kGroups + g; tile * kRows < n && ok;
-         tile += (long long)gridDim.x * kGroups) {
+    const uint32_t bar = smem_addr(gs + S::Bar), bar_in = bar + 8u;
+    uint32_t phase = 0u, phase_in = 0u;
+    bool ok = true, loading = false;
+    float* xs = reinterpret_cast<float*>(gs + S::XS);
+    float* zs = reinterpret_cast<float*>(gs + S::H);
+    const float* b3 = reinterpret_cast<const float*>(sm + S::Bias) + 2 * kH;
+    const long long stride = (long long)gridDim.x * kFwdGroups;
+    // a whole tile's inputs, 3 KB in a row: one bulk copy (row0 * 24 bytes is
+    // a multiple of 16 when row0 is one of 128)
+    auto whole = [&](long long tile) { return (tile + 1) * kRows <= n; };
+    long long tile = (long long)blockIdx.x * kFwdGroups + g;
+    if (whole(tile)) {
+        if (r == 0) bulk_load(smem_addr(xs), x + kIn * kRows * tile, kRows * kIn * 4, bar_in);
+        loading = true;
+    }
+    for (; tile * kRows < n; tile += stride) {
         const long long row0 = tile * kRows;
         const int rows = (int)min((long long)kRows, n - row0);
-        // the tile's inputs, rows x 6 contiguous floats: coalesced 16-byte loads
-        // (row0 * 24 bytes is a multiple of 16 when row0 is a multiple of 128)
-        const float4* xg = reinterpret_cast<const float4*>(x + kIn * row0);
-        const int nx = rows * kIn;
-        for (int i = r; i < (nx >> 2); i += kRows) reinterpret_cast<float4*>(xs)[i] = __ldg(xg + i);
-        for (int i = (nx & ~3) + r; i < nx; i += kRows) xs[i] = __ldg(x + kIn * row0 + i);
-        group_sync(g);
         float f[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-        if (r < rows) {
+        if (loading) {
+            ok = mbar_wait(bar_in, phase_in) && ok;
+            phase_in ^= 1u;
+            loading = false;
 #pragma unroll
             for (int k = 0; k < 6; ++k) f[k] = xs[kIn * r + k];
-        }
-        store_input_row(gs + FwdSmem::X, r, f);
-        ok = forward_tile(sm, gs, tcol, t_row, net, bar, phase, r, g);
-        if (!ok) break;
-        float zz[kOutPad];
-        output_epilogue(t_row, net.params + ob3, zz);
-        // outputs through shared memory (h2 is consumed): rows x 45 contiguous
-        // floats leave with coalesced 16-byte stores (row0 * 180 bytes is a
-        // multiple of 16)
+        } else if (r < rows) {
 #pragma unroll
-        for (int j = 0; j < kOut; ++j) zs[kOut * r + j] = zz[j];
-        group_sync(g);
-        float4* zg = reinterpret_cast<float4*>(z + kOut * row0);
-        const int nz = rows * kOut;
-        for (int i = r; i < (nz >> 2); i += kRows) zg[i] = reinterpret_cast<const float4*>(zs)[i];
-        for (int i = (nz & ~3) + r; i < nz; i += kRows) z[kOut * row0 + i] = zs[i];
+            for (int k = 0; k < 6; ++k) f[k] = __ldg(x + kIn * (row0 + r) + k);
+        }
+        store_input_row(gs + S::X, r, f);
+        if (r == 0) bulk_store_wait_read();         // the last outputs have left the staging tile
+        fence_async_smem();
         tc_fence_before();
-        group_sync(g);
+        ok = group_sync_and(g, ok);                 // publishes X; the group agrees on the waits so far
+        if (!ok) break;
+        loading = whole(tile + stride);
+        if (loading && r == 0)
+            bulk_load(smem_addr(xs), x + kIn * kRows * (tile + stride), kRows * kIn * 4, bar_in);
+        forward_tile<S>(sm, gs, tcol, t_row, phase, r, g, ok);
+        // outputs through shared memory (h2 is consumed): rows x 45 contiguous
+        // floats (row0 * 180 bytes is a multiple of 16)
+        float v[32], u[16];
+        tmem_ld32(t_row, v);
+        tmem_ld16(t_row + 32u, u);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) zs[kOut * r + j] = v[j] + b3[j];
+#pragma unroll
+        for (int j = 32; j < kOut; ++j) zs[kOut * r + j] = u[j - 32] + b3[j];
+        publish_group(g);
+        if (rows == kRows) {
+            if (r == 0) bulk_store(z + kOut * row0, smem_addr(zs), kRows * kOut * 4);
+        } else {
+            for (int i = r; i < rows * kOut; i += kRows) z[kOut * row0 + i] = zs[i];
+        }
     }
-    fwd_epilogue_free(sm, tbase, bar, phase, ok, net);
+    if (!ok && loading) (void)mbar_wait(bar_in, phase_in);     // a copy in flight ends before the memory is given back
+    if (r == 0) bulk_store_wait();
+    fwd_epilogue_free<S>(sm, tbase, bar, phase, ok, net);
 }
 
 // Draw of one query from the network output z (see the sampler in the oracle):
@@ -523,25 +601,27 @@ __device__ __forceinline__ bool sample_exit(const float (&z)[kOutPad], uint4 ua,
     return trans;
 }
 
-__global__ void __launch_bounds__(kFwdThreads, 1) k_sur_infer(const SurNet net, const TransportParams P)
+__global__ void __launch_bounds__(kInferGroups * kRows, 1) k_sur_infer(const SurNet net, const TransportParams P)
 {
+    using S = InferS;
     extern __shared__ __align__(1024) unsigned char sm[];
     uint32_t tbase;
-    fwd_prologue(sm, net, tbase);
+    fwd_prologue<S, kInferGroups>(sm, net, tbase);
     const int g = threadIdx.x / kRows, r = threadIdx.x % kRows;
     const int lane = r & 31;
-    unsigned char* gs = sm + FwdSmem::G0 + g * FwdSmem::GBytes;
+    unsigned char* gs = sm + S::G0 + g * S::GBytes;
     const uint32_t tcol = tbase + (uint32_t)(g * kRows);
     const uint32_t t_row = tcol + ((uint32_t)((r >> 5) * 32) << 16);
-    const uint32_t bar = smem_addr(gs + FwdSmem::Bar);
+    const uint32_t bar = smem_addr(gs + S::Bar);
+    const float* b3 = reinterpret_cast<const float*>(sm + S::Bias) + 2 * kH;
     uint32_t phase = 0u;
     bool ok = true;
     const long long nq = min((long long)*P.sq_count, P.sq_cap);
     unsigned long long acc_ap = 0ull;
-    SurQuery* qs = reinterpret_cast<SurQuery*>(gs + FwdSmem::QS);
+    SurQuery* qs = reinterpret_cast<SurQuery*>(gs + S::QS);
     static_assert(sizeof(SurQuery) % 16 == 0, "query records are copied in 16-byte pieces");
-    for (long long tile = (long long)blockIdx.x * kGroups + g; tile * kRows < nq && ok;
-         tile += (long long)gridDim.x * kGroups) {
+    for (long long tile = (long long)blockIdx.x * kInferGroups + g; tile * kRows < nq;
+         tile += (long long)gridDim.x * kInferGroups) {
         const long long row = tile * kRows + r;
         const int rows = (int)min((long long)kRows, nq - tile * kRows);
         // the tile's query records, contiguous: coalesced 16-byte loads
@@ -557,13 +637,14 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sur_infer(const SurNet net, 
 #pragma unroll
             for (int k = 0; k < 6; ++k) f[k] = qs[r].x[k];
         }
-        store_input_row(gs + FwdSmem::X, r, f);
-        ok = forward_tile(sm, gs, tcol, t_row, net, bar, phase, r, g);
-        if (!ok) break;
+        store_input_row(gs + S::X, r, f);
+        publish_group(g);
+        forward_tile<S>(sm, gs, tcol, t_row, phase, r, g, ok);
         float zz[kOutPad];
-        output_epilogue(t_row, net.params + ob3, zz);
+        output_epilogue(t_row, b3, zz);
         tc_fence_before();
-        group_sync(g);
+        ok = group_sync_and(g, ok);
+        if (!ok) break;
 
         bool emit = false;
         PhaseRec rec;
@@ -665,7 +746,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sur_infer(const SurNet net, 
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) acc_ap += __shfl_xor_sync(kFull, acc_ap, o);
     if (lane == 0 && acc_ap) atomicAdd(P.stats + kStAp, acc_ap);
-    fwd_epilogue_free(sm, tbase, bar, phase, ok, net);
+    fwd_epilogue_free<S>(sm, tbase, bar, phase, ok, net);
 }
 
 // ============================================================================
@@ -760,10 +841,14 @@ __global__ void __launch_bounds__(kRows, 1) k_sur_train(const SurNet net, const 
 {
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ float s_db3[kOutPad];              // the CTA's b3 gradient
+    __shared__ float s_b3[kOutPad];
     const uint32_t s0 = smem_addr(sm);
     const int r = threadIdx.x;
     const int lane = r & 31;
-    if (r < kOutPad) s_db3[r] = 0.0f;
+    if (r < kOutPad) {
+        s_db3[r] = 0.0f;
+        s_b3[r] = r < kOut ? net.params[ob3 + r] : 0.0f;
+    }
     copy_to_smem(sm + TrainSmem::Img, net.img, kImgBytes);
     zero_smem(sm + TrainSmem::XT, kInPad * kRows * 2);
     zero_smem(sm + TrainSmem::Bt + kmaj(128, 0, kRows), 16 * kRows * 2);
@@ -829,7 +914,7 @@ __global__ void __launch_bounds__(kRows, 1) k_sur_train(const SurNet net, const 
         }
         if (!(ok = complete(bar, phase))) break;
         float zz[kOutPad], g[kOutPad];
-        output_epilogue(t_row, net.params + ob3, zz);
+        output_epilogue(t_row, s_b3, zz);
         float lrow = 0.0f;
         if (valid) {
             lrow = row_loss_grad(zz, label[row] > 0 ? 1.0f : 0.0f, yt + 5 * row, g);
@@ -1023,7 +1108,7 @@ __global__ void k_sur_adam(const SurNet net, float lr, float c1, float c2, int p
 
 }  // namespace
 
-size_t sur_forward_smem_bytes() { return FwdSmem::Bytes; }
+size_t sur_forward_smem_bytes() { return std::max(FwdS::Bytes, InferS::Bytes); }
 size_t sur_train_smem_bytes() { return TrainSmem::Bytes; }
 
 cudaError_t launch_sur_pack(const SurNet& net, cudaStream_t s)
@@ -1036,14 +1121,14 @@ cudaError_t launch_sur_forward(const SurNet& net, const float* x, long long n, f
 {
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_sur_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem::Bytes);
+        cudaError_t e = cudaFuncSetAttribute(k_sur_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdS::Bytes);
         if (e != cudaSuccess) return e;
         attr = true;
     }
     if (n <= 0) return cudaSuccess;
     const long long tiles = (n + kRows - 1) / kRows;
-    const long long ctas = (tiles + kGroups - 1) / kGroups;
-    k_sur_forward<<<(int)std::min<long long>(ctas, grid), kFwdThreads, FwdSmem::Bytes, s>>>(net, x, n, z);
+    const long long ctas = (tiles + kFwdGroups - 1) / kFwdGroups;
+    k_sur_forward<<<(int)std::min<long long>(ctas, grid), kFwdGroups * kRows, FwdS::Bytes, s>>>(net, x, n, z);
     return cudaGetLastError();
 }
 
@@ -1051,11 +1136,11 @@ cudaError_t launch_sur_infer(const SurNet& net, const TransportParams& p, int gr
 {
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_sur_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem::Bytes);
+        cudaError_t e = cudaFuncSetAttribute(k_sur_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, InferS::Bytes);
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    k_sur_infer<<<grid, kFwdThreads, FwdSmem::Bytes, s>>>(net, p);
+    k_sur_infer<<<grid, kInferGroups * kRows, InferS::Bytes, s>>>(net, p);
     return cudaGetLastError();
 }
 
