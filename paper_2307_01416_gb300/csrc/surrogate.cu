@@ -28,7 +28,34 @@ namespace {
 using namespace dev;
 using namespace sur;
 
-constexpr int kRows = 128;                // rows (tracks) per tile, one thread each
+constexpr int kRows = 128;                // rows (tracks) per tile
+
+// Output rows in the training kernel's order (W3P): one 16-row block per
+// mixture component -- the transmission logit (component 0), its mixture
+// logit, 5 means, 5 log widths, padding -- so that a component's outputs are
+// 16 aligned accumulator columns.
+__host__ __device__ constexpr int w3p_row(int o)
+{
+    if (o == 0) return 0;
+    if (o < 1 + kNComp) return 16 * (o - 1) + 1;
+    const int k = (o - 5) % 20, c = k / kDY, j = k % kDY;
+    return 16 * c + (o < 25 ? 2 : 7) + j;
+}
+__host__ __device__ constexpr int w3p_output(int row)      // -1: padding
+{
+    const int c = row / 16, j = row % 16;
+    if (j == 0) return c == 0 ? 0 : -1;
+    if (j == 1) return 1 + c;
+    if (j < 7) return 5 + kDY * c + (j - 2);
+    return j < 12 ? 25 + kDY * c + (j - 7) : -1;
+}
+constexpr bool w3p_is_inverse()
+{
+    for (int o = 0; o < kOut; ++o)
+        if (w3p_output(w3p_row(o)) != o) return false;
+    return true;
+}
+static_assert(w3p_is_inverse(), "the training order holds every output");
 constexpr int kWaitLimit = 1 << 22;       // mbarrier polls before a wait is declared failed
 
 // Byte offset of element (r, k) of an R x K operand in the no-swizzle
@@ -199,6 +226,30 @@ __device__ __forceinline__ void mma_tile(uint32_t d_tmem, uint32_t a_saddr, uint
     }
 }
 
+// One operand of a tile GEMM in shared memory, stored as kmaj(row, column,
+// columns).  K-major: rows are M or N, columns K.  MN-major (the transposed
+// operand, without a transposed copy): rows are K, columns M or N; a core
+// matrix then holds 8 K rows of 8 contiguous M or N values.
+struct Operand {
+    uint32_t saddr;
+    int cols;
+    bool mn_major;
+};
+
+// D[128 x N] (+)= A B^T over K, either operand K-major or MN-major.
+__device__ __forceinline__ void mma_operands(uint32_t d_tmem, Operand A, Operand B, int K, int N, bool accumulate)
+{
+    const uint32_t idesc = idesc_bf16(kRows, N) | (A.mn_major ? 1u << 15 : 0u) | (B.mn_major ? 1u << 16 : 0u);
+    const uint32_t ra = (uint32_t)(A.cols >> 3) << 7, rb = (uint32_t)(B.cols >> 3) << 7;   // 8 rows
+    for (int kc = 0; kc < (K >> 4); ++kc) {
+        const uint64_t a = A.mn_major ? sdesc(A.saddr + (uint32_t)kc * 2u * ra, ra, 128u)
+                                      : sdesc(A.saddr + (uint32_t)kc * 256u, 128u, ra);
+        const uint64_t b = B.mn_major ? sdesc(B.saddr + (uint32_t)kc * 2u * rb, rb, 128u)
+                                      : sdesc(B.saddr + (uint32_t)kc * 256u, 128u, rb);
+        umma(d_tmem, a, b, idesc, (accumulate || kc > 0) ? 1u : 0u);
+    }
+}
+
 // Make this thread's generic-proxy shared-memory writes and tensor-memory
 // reads visible to the next tensor-core operation, then synchronise.
 __device__ __forceinline__ void publish()
@@ -206,17 +257,6 @@ __device__ __forceinline__ void publish()
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
-}
-
-// Wait (all threads) for the tensor-core work committed to mbar; the CTA
-// agrees on the outcome.
-__device__ __forceinline__ bool complete(uint32_t mbar, uint32_t& phase)
-{
-    const bool ok = mbar_wait(mbar, phase);
-    phase ^= 1u;
-    const bool all = __syncthreads_and(ok) != 0;
-    tc_fence_after();
-    return all;
 }
 
 // Barrier of one 128-thread warpgroup (named barrier 1 + g): the forward
@@ -251,12 +291,6 @@ __device__ __forceinline__ void copy_to_smem(unsigned char* dst, const unsigned 
     const uint4* s = reinterpret_cast<const uint4*>(src);
     uint4* d = reinterpret_cast<uint4*>(dst);
     for (int i = threadIdx.x; i < (bytes >> 4); i += blockDim.x) d[i] = __ldg(s + i);
-}
-
-__device__ __forceinline__ void zero_smem(unsigned char* dst, int bytes)
-{
-    uint4* d = reinterpret_cast<uint4*>(dst);
-    for (int i = threadIdx.x; i < (bytes >> 4); i += blockDim.x) d[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // Row r of a [128 x 16] input tile: the 6 features, then zeros.
@@ -339,32 +373,6 @@ __device__ __forceinline__ void hidden_epilogue_fwd(uint32_t t_row, const float*
     tmem_cols_pipelined(t_row, kH, [&](const uint32_t (&v)[16], int c0) { relu_pack16(v, bias, c0, dst, r); });
 }
 
-// Hidden-layer epilogue of training: relu(D + b) to BF16 into the K-major
-// tile dst and its transposed copy dstT (rows = units, K = tile rows), and the
-// ReLU mask (bit c of mask[c / 32]: D + b > 0; the caller zeroes mask).
-__device__ __forceinline__ void hidden_epilogue_train(uint32_t t_row, const float* __restrict__ bias,
-                                                      unsigned char* dst, unsigned char* dstT, int r,
-                                                      uint32_t (&mask)[4])
-{
-    tmem_cols_pipelined(t_row, kH, [&](const uint32_t (&v)[16], int c0) {
-        uint32_t w[8];
-        uint32_t mbits = 0u;
-#pragma unroll
-        for (int j = 0; j < 16; j += 2) {
-            const float a0 = __uint_as_float(v[j]) + __ldg(bias + c0 + j);
-            const float a1 = __uint_as_float(v[j + 1]) + __ldg(bias + c0 + j + 1);
-            mbits |= (a0 > 0.0f ? 1u : 0u) << j;
-            mbits |= (a1 > 0.0f ? 1u : 0u) << (j + 1);
-            w[j >> 1] = pack_bf16(fmaxf(a0, 0.0f), fmaxf(a1, 0.0f));
-            *reinterpret_cast<unsigned short*>(dstT + kmaj(c0 + j, r, kRows)) = (unsigned short)(w[j >> 1] & 0xFFFFu);
-            *reinterpret_cast<unsigned short*>(dstT + kmaj(c0 + j + 1, r, kRows)) = (unsigned short)(w[j >> 1] >> 16);
-        }
-        *reinterpret_cast<uint4*>(dst + kmaj(r, c0, kH)) = make_uint4(w[0], w[1], w[2], w[3]);
-        *reinterpret_cast<uint4*>(dst + kmaj(r, c0 + 8, kH)) = make_uint4(w[4], w[5], w[6], w[7]);
-        mask[c0 >> 5] |= mbits << (c0 & 31);
-    });
-}
-
 // z = D3 + b3 for row r (48 columns, 45 used; b3 in shared memory, padded with zeros).
 __device__ __forceinline__ void output_epilogue(uint32_t t_d3, const float* b3, float (&z)[kOutPad])
 {
@@ -399,7 +407,7 @@ __device__ __forceinline__ void output_epilogue(uint32_t t_d3, const float* b3, 
 template <int kG, bool kQueries>
 struct FwdSmem {
     static constexpr int W = 0;                                   // W1, W2, W3 images
-    static constexpr int Bias = kImgW2T;                          // b1, b2, b3 (padded), FP32
+    static constexpr int Bias = kImgW3P;                          // b1, b2, b3 (padded), FP32
     static constexpr int G0 = (Bias + (2 * kH + kOutPad) * 4 + 127) / 128 * 128;     // the groups' regions
     // offsets within a group's region
     static constexpr int X = 0;                                   // [128 x 16]
@@ -460,7 +468,7 @@ __device__ __forceinline__ void forward_tile(unsigned char* sm, unsigned char* g
 template <class S, int kG>
 __device__ __forceinline__ void fwd_prologue(unsigned char* sm, const SurNet& net, uint32_t& tbase)
 {
-    copy_to_smem(sm + S::W, net.img, kImgW2T);
+    copy_to_smem(sm + S::W, net.img, kImgW3P);
     float* bias = reinterpret_cast<float*>(sm + S::Bias);
     for (int i = threadIdx.x; i < 2 * kH + kOutPad; i += blockDim.x)
         bias[i] = i < kH ? net.params[ob1 + i]
@@ -753,20 +761,37 @@ __global__ void __launch_bounds__(kInferGroups * kRows, 1) k_sur_infer(const Sur
 // Training: forward, loss, backward and weight-gradient accumulation of the
 // CTA's tiles in one kernel.
 // ============================================================================
+// A batch of 16,384 rows is 128 tiles, one per CTA, so a launch lasts as long
+// as one tile's chain of six GEMM phases, the loss between them, the operand
+// load before and the gradient store after it: latency, not the tensor core
+// (1 us of work).  What shortens the chain: 512 threads, four per row, each
+// taking 32 columns of every epilogue and one mixture component of the loss;
+// weight images by bulk copies while the inputs are read; one operand tile
+// per activation, read K-major by the forward GEMMs and MN-major by the weight
+// gradients and the backward ones (no transposed copies: 2-byte stores with
+// 4-way bank conflicts); the b3 gradient by one butterfly per component.
+// 20.7 us a launch; 40.8 us with 128 threads and transposed copies.
+constexpr int kTrainThreads = 512;
+constexpr int kH1Cols = kH + 16;             // h1 and the all-ones column (b2 gradient)
 struct TrainSmem {
-    static constexpr int Img = 0;                                  // all five weight images
-    static constexpr int X = kImgBytes;                            // [128 x 16]
-    static constexpr int XT = X + kRows * kInPad * 2;              // [16 x 128]: features, row 6 = ones
-    static constexpr int A = XT + kInPad * kRows * 2;              // [128 x 128]: h1, h2, then da2
-    static constexpr int Bt = A + kRows * kH * 2;                  // [144 x 128]: h1^T, row 128 = ones
-    static constexpr int C = Bt + 144 * kRows * 2;                 // [128 x 128]: h2^T, da2^T, da1^T
-    static constexpr int DZ = C + kH * kRows * 2;                  // [128 x 48]
-    static constexpr int DZT = DZ + kRows * kOutPad * 2;           // [48 x 128]
-    static constexpr int Bar = DZT + kOutPad * kRows * 2;
-    static constexpr int Slot = Bar + 8;
+    static constexpr int Img = 0;                                  // W1, W2, W3 images
+    static constexpr int W3P = kImgW3P;                            // W3 with one 16-row block per component
+    static constexpr int X = kImgBytes;                            // [128 x 16]: features, column 6 = ones (b1 gradient)
+    static constexpr int H1 = X + kRows * kInPad * 2;              // [128 x 144]: h1, ones
+    static constexpr int H2 = H1 + kRows * kH1Cols * 2;            // [128 x 128]: h2, then da2, then da1
+    static constexpr int DZ = H2 + kRows * kH * 2;                 // [128 x 48]
+    static constexpr int B1 = DZ + kRows * kOutPad * 2;            // biases (b3 in W3P's order)
+    static constexpr int B2 = B1 + kH * 4;
+    static constexpr int B3 = B2 + kH * 4;
+    static constexpr int Alpha = B3 + kOutP * 4;                   // [128 x 4]: mixture logits of the tile
+    static constexpr int Lc = Alpha + kRows * kNComp * 4;          // [128 x 4]: component log densities
+    static constexpr int Db3 = Lc + kRows * kNComp * 4;            // [4 warps x 48] row sums, then [48] over the tiles
+    static constexpr int Bar = Db3 + 5 * kOutPad * 4;
+    static constexpr int Slot = Bar + 16;
     static constexpr int Bytes = Slot + 8;
 };
 static_assert(TrainSmem::Bytes <= 232448, "training tile exceeds the shared memory of one CTA");
+static_assert(TrainSmem::Bar % 16 == 0 && kImgW3P % 128 == 0 && kImgBytes % 128 == 0, "alignment");
 // tensor-memory columns: D1/D3/D4 at 0, D2/D5 at 128, dW2 (with db2) at 256,
 // dW3^T at 400, dW1 (with db1) at 448
 constexpr uint32_t kTrainCols = 512, kColW2 = 256, kColW3T = 400, kColW1 = 448;
@@ -778,273 +803,335 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
-// Loss of one row and its gradient with respect to z (written out from the
-// loss: BCE of the transmission logit plus, for transmitted tracks, the
-// negative log-likelihood of the mixture).
-__device__ __forceinline__ float row_loss_grad(const float (&z)[kOutPad], float t, const float* __restrict__ yv,
-                                               float (&g)[kOutPad])
+// relu(D + b) of this thread's 32 columns [c0, c0 + 32) of row r to BF16 into
+// the tile dst of `cols` columns; returns the ReLU mask (bit j: D + b > 0).
+__device__ __forceinline__ uint32_t hidden_epilogue_train(uint32_t t_row, const float* bias, unsigned char* dst, int cols,
+                                                          int r, int c0)
 {
+    uint32_t mask = 0u;
+    tmem_cols_pipelined(t_row + (uint32_t)c0, 32, [&](const uint32_t (&v)[16], int k0) {
+        uint32_t w[8];
 #pragma unroll
-    for (int j = 0; j < kOutPad; ++j) g[j] = 0.0f;
-    const float logit = z[0];
-    const float sig = 1.0f / (1.0f + expf(-logit));
-    g[0] = sig - t;
-    float loss = fmaxf(logit, 0.0f) + log1pf(expf(-fabsf(logit))) - t * logit;
-    if (t > 0.0f) {
-        float y[kDY];
+        for (int j = 0; j < 16; j += 4) {
+            const float4 b = *reinterpret_cast<const float4*>(bias + c0 + k0 + j);
+            const float2 p = add2(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), b.x, b.y);
+            const float2 q = add2(__uint_as_float(v[j + 2]), __uint_as_float(v[j + 3]), b.z, b.w);
+            mask |= (p.x > 0.0f ? 1u : 0u) << (k0 + j);
+            mask |= (p.y > 0.0f ? 1u : 0u) << (k0 + j + 1);
+            mask |= (q.x > 0.0f ? 1u : 0u) << (k0 + j + 2);
+            mask |= (q.y > 0.0f ? 1u : 0u) << (k0 + j + 3);
+            w[j >> 1] = relu_bf16x2(pack_bf16(p.x, p.y));
+            w[(j >> 1) + 1] = relu_bf16x2(pack_bf16(q.x, q.y));
+        }
+        *reinterpret_cast<uint4*>(dst + kmaj(r, c0 + k0, cols)) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(dst + kmaj(r, c0 + k0 + 8, cols)) = make_uint4(w[4], w[5], w[6], w[7]);
+    });
+    return mask;
+}
+
+// D masked by the ReLU's derivative, this thread's 32 columns of row r to BF16.
+__device__ __forceinline__ void masked_epilogue(uint32_t t_row, uint32_t mask, unsigned char* dst, int r, int c0)
+{
+    tmem_cols_pipelined(t_row + (uint32_t)c0, 32, [&](const uint32_t (&v)[16], int k0) {
+        uint32_t w[8];
 #pragma unroll
-        for (int j = 0; j < kDY; ++j) y[j] = yv[j];
-        const float amax = fmaxf(fmaxf(z[1], z[2]), fmaxf(z[3], z[4]));
+        for (int j = 0; j < 16; j += 2) {
+            const float a0 = ((mask >> (k0 + j)) & 1u) ? __uint_as_float(v[j]) : 0.0f;
+            const float a1 = ((mask >> (k0 + j + 1)) & 1u) ? __uint_as_float(v[j + 1]) : 0.0f;
+            w[j >> 1] = pack_bf16(a0, a1);
+        }
+        *reinterpret_cast<uint4*>(dst + kmaj(r, c0 + k0, kH)) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(dst + kmaj(r, c0 + k0 + 8, kH)) = make_uint4(w[4], w[5], w[6], w[7]);
+    });
+}
+
+// cols consecutive accumulator columns of this thread's row as floats at dst.
+template <int kCols>
+__device__ __forceinline__ void store_partial(uint32_t taddr, bool have, float* dst)
+{
+    uint32_t v[16];
+#pragma unroll
+    for (int c0 = 0; c0 < kCols; c0 += 16) {
+        if (have) {
+            tmem_ld16_async(taddr + (uint32_t)c0, v);
+            tmem_wait16(v);
+        }
+#pragma unroll
+        for (int j = 0; j < 16 && c0 + j < kCols; ++j) dst[c0 + j] = have ? __uint_as_float(v[j]) : 0.0f;
+    }
+}
+
+__global__ void __launch_bounds__(kTrainThreads, 1) k_sur_train(const SurNet net, const float* __restrict__ x,
+                                                                const float* __restrict__ yt,
+                                                                const int* __restrict__ label, long long first,
+                                                                long long rows, long long n, float inv_rows)
+{
+    using S = TrainSmem;
+    extern __shared__ __align__(1024) unsigned char sm[];
+    const uint32_t s0 = smem_addr(sm);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int q = warp & 3, cg = warp >> 2;       // row quarter (tensor-memory lanes), column group / component
+    const int r = q * 32 + lane;
+    const uint32_t bar = s0 + S::Bar, bar_img = bar + 8u;
+    if (threadIdx.x == 0) {
+        mbar_init(bar);
+        mbar_init(bar_img);
+        bulk_load(s0 + S::Img, net.img, kImgBytes, bar_img);
+    }
+    float* b1 = reinterpret_cast<float*>(sm + S::B1);
+    float* b2 = reinterpret_cast<float*>(sm + S::B2);
+    float* b3 = reinterpret_cast<float*>(sm + S::B3);
+    float* s_alpha = reinterpret_cast<float*>(sm + S::Alpha);
+    float* s_lc = reinterpret_cast<float*>(sm + S::Lc);
+    float* s_red = reinterpret_cast<float*>(sm + S::Db3);
+    float* s_db3 = s_red + 4 * kOutPad;
+    if (threadIdx.x < kH) b1[threadIdx.x] = net.params[ob1 + threadIdx.x];
+    else if (threadIdx.x < 2 * kH) b2[threadIdx.x - kH] = net.params[ob2 + threadIdx.x - kH];
+    else if (threadIdx.x < 2 * kH + kOutP) {
+        const int o = w3p_output(threadIdx.x - 2 * kH);
+        b3[threadIdx.x - 2 * kH] = o >= 0 ? net.params[ob3 + o] : 0.0f;
+    }
+    if (threadIdx.x < kOutPad) s_db3[threadIdx.x] = 0.0f;
+    // constant operand columns: h1's ones, dz's padding
+    if (cg == 0) {
+        *reinterpret_cast<uint4*>(sm + S::H1 + kmaj(r, kH, kH1Cols)) = make_uint4(0x3F80u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(sm + S::H1 + kmaj(r, kH + 8, kH1Cols)) = make_uint4(0u, 0u, 0u, 0u);
+    } else if (cg == 1) {
+        *reinterpret_cast<uint4*>(sm + S::DZ + kmaj(r, kOutPad - 8, kOutPad)) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (warp == 0) tmem_alloc(s0 + S::Slot, kTrainCols);
+    fence_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tbase = *reinterpret_cast<volatile uint32_t*>(sm + S::Slot);
+    const uint32_t t_row = tbase + ((uint32_t)(q * 32) << 16);
+    const int c0 = 32 * cg;
+    uint32_t phase = 0u;
+    bool ok = mbar_wait(bar_img, 0u);
+    int tiles_done = 0;
+    double loss_acc = 0.0;
+    const long long end = min(first + rows, n);
+    // operands K-major (K) and MN-major (M)
+    const Operand xK{s0 + S::X, kInPad, false}, h1K{s0 + S::H1, kH1Cols, false}, h2K{s0 + S::H2, kH, false},
+        dzK{s0 + S::DZ, kOutPad, false};
+    const Operand xM{s0 + S::X, kInPad, true}, h1M{s0 + S::H1, kH1Cols, true}, h2M{s0 + S::H2, kH, true},
+        dzM{s0 + S::DZ, kOutPad, true};
+    const Operand w1K{s0 + S::Img + kImgW1, kInPad, false}, w2K{s0 + S::Img + kImgW2, kH, false},
+        w3pK{s0 + S::W3P, kH, false};
+    const Operand w2M{s0 + S::Img + kImgW2, kH, true}, w3M{s0 + S::Img + kImgW3, kH, true};
+    auto step = [&]() {                             // the tensor core's work committed last
+        const bool done = mbar_wait(bar, phase);
+        phase ^= 1u;
+        tc_fence_after();
+        return done;
+    };
+    for (long long tile = blockIdx.x; first + tile * kRows < end; tile += gridDim.x) {
+        const long long row = first + tile * kRows + r;
+        const bool valid = row < end;
+        // ---- inputs ----
+        if (cg == 0) {
+            float f[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+            if (valid) {
+#pragma unroll
+                for (int k = 0; k < 6; ++k) f[k] = __ldg(x + 6 * row + k);
+            }
+            *reinterpret_cast<uint4*>(sm + S::X + kmaj(r, 0, kInPad)) =
+                make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), 0x3F80u);
+            *reinterpret_cast<uint4*>(sm + S::X + kmaj(r, 8, kInPad)) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        float y[kDY] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        float t = 0.0f;
+        if (valid) {
+            t = __ldg(label + row) > 0 ? 1.0f : 0.0f;
+#pragma unroll
+            for (int j = 0; j < kDY; ++j) y[j] = __ldg(yt + 5 * row + j);
+        }
+        // ---- layer 1 (the CTA agrees here on the waits so far) ----
+        fence_async_smem();
+        tc_fence_before();
+        if (!__syncthreads_and(ok)) {
+            ok = false;
+            break;
+        }
+        if (threadIdx.x == 0) {
+            tc_fence_after();
+            mma_operands(tbase, xK, w1K, kInPad, kH, false);
+            umma_commit(bar);
+        }
+        ok = step() && ok;
+        const uint32_t m1 = hidden_epilogue_train(t_row, b1, sm + S::H1, kH1Cols, r, c0);
+        // ---- layer 2 ----
+        publish();
+        if (threadIdx.x == 0) {
+            tc_fence_after();
+            mma_operands(tbase + 128u, h1K, w2K, kH, kH, false);
+            umma_commit(bar);
+        }
+        ok = step() && ok;
+        const uint32_t m2 = hidden_epilogue_train(t_row + 128u, b2, sm + S::H2, kH, r, c0);
+        // ---- output layer: component cg's 16 columns ----
+        publish();
+        if (threadIdx.x == 0) {
+            tc_fence_after();
+            mma_operands(tbase, h2K, w3pK, kH, kOutP, false);
+            umma_commit(bar);
+        }
+        ok = step() && ok;
+        // loss of the row and its gradient with respect to z (BCE of the
+        // transmission logit plus, for transmitted tracks, the negative
+        // log-likelihood of the mixture); this thread has component cg
+        float zv[16];
+        tmem_ld16(t_row + (uint32_t)(16 * cg), zv);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) zv[j] += b3[16 * cg + j];
+        const float alpha = zv[1];
+        s_alpha[kNComp * r + cg] = alpha;
+        __syncthreads();
+        const float4 al = *reinterpret_cast<const float4*>(s_alpha + kNComp * r);
+        const float za[kNComp] = {al.x, al.y, al.z, al.w};
+        const float amax = fmaxf(fmaxf(za[0], za[1]), fmaxf(za[2], za[3]));
         float asum = 0.0f;
 #pragma unroll
-        for (int c = 0; c < kNComp; ++c) asum += expf(z[1 + c] - amax);
+        for (int c = 0; c < kNComp; ++c) asum += expf(za[c] - amax);
         const float lse_a = amax + logf(asum);
-        float lc[kNComp];
+        float acc = alpha - lse_a;
 #pragma unroll
-        for (int c = 0; c < kNComp; ++c) {
-            float acc = z[1 + c] - lse_a;
-#pragma unroll
-            for (int j = 0; j < kDY; ++j) {
-                const float s = z[25 + 5 * c + j];
-                const float rr = (y[j] - z[5 + 5 * c + j]) * expf(-s);
-                acc += -0.5f * rr * rr - s - 0.91893853320467274f;
-            }
-            lc[c] = acc;
+        for (int j = 0; j < kDY; ++j) {
+            const float s = zv[7 + j];
+            const float rr = (y[j] - zv[2 + j]) * expf(-s);
+            acc += -0.5f * rr * rr - s - 0.91893853320467274f;
         }
+        s_lc[kNComp * r + cg] = acc;
+        __syncthreads();
+        const float4 l4 = *reinterpret_cast<const float4*>(s_lc + kNComp * r);
+        const float lc[kNComp] = {l4.x, l4.y, l4.z, l4.w};
         const float lmax = fmaxf(fmaxf(lc[0], lc[1]), fmaxf(lc[2], lc[3]));
         float lsum = 0.0f;
 #pragma unroll
         for (int c = 0; c < kNComp; ++c) lsum += expf(lc[c] - lmax);
         const float L = lmax + logf(lsum);
-        loss -= L;
+        // gradient: 0 logit (component 0's thread), 1 mixture logit, 2.. means, 7.. log widths
+        float g[12];
 #pragma unroll
-        for (int c = 0; c < kNComp; ++c) {
-            const float resp = expf(lc[c] - L);
-            const float pi = expf(z[1 + c] - lse_a);
-            g[1 + c] = pi - resp;
-#pragma unroll
-            for (int j = 0; j < kDY; ++j) {
-                const float s = z[25 + 5 * c + j];
-                const float inv2 = expf(-2.0f * s);
-                const float diff = y[j] - z[5 + 5 * c + j];
-                g[5 + 5 * c + j] = -resp * diff * inv2;
-                g[25 + 5 * c + j] = -resp * (diff * diff * inv2 - 1.0f);
+        for (int j = 0; j < 12; ++j) g[j] = 0.0f;
+        if (valid) {
+            if (cg == 0) {
+                const float logit = zv[0];
+                const float sig = 1.0f / (1.0f + expf(-logit));
+                g[0] = sig - t;
+                float loss = fmaxf(logit, 0.0f) + log1pf(expf(-fabsf(logit))) - t * logit;
+                if (t > 0.0f) loss -= L;
+                loss_acc += (double)loss;
             }
-        }
-    }
-    return loss;
-}
-
-__global__ void __launch_bounds__(kRows, 1) k_sur_train(const SurNet net, const float* __restrict__ x,
-                                                        const float* __restrict__ yt, const int* __restrict__ label,
-                                                        long long first, long long rows, long long n, float inv_rows)
-{
-    extern __shared__ __align__(1024) unsigned char sm[];
-    __shared__ float s_db3[kOutPad];              // the CTA's b3 gradient
-    __shared__ float s_b3[kOutPad];
-    const uint32_t s0 = smem_addr(sm);
-    const int r = threadIdx.x;
-    const int lane = r & 31;
-    if (r < kOutPad) {
-        s_db3[r] = 0.0f;
-        s_b3[r] = r < kOut ? net.params[ob3 + r] : 0.0f;
-    }
-    copy_to_smem(sm + TrainSmem::Img, net.img, kImgBytes);
-    zero_smem(sm + TrainSmem::XT, kInPad * kRows * 2);
-    zero_smem(sm + TrainSmem::Bt + kmaj(128, 0, kRows), 16 * kRows * 2);
-    zero_smem(sm + TrainSmem::DZT, kOutPad * kRows * 2);
-    __syncthreads();
-    // constant operand rows: XT row 6 and h1^T row 128 are all ones (bias gradients)
-    {
-        const unsigned short one = bf16_bits(1.0f);
-        *reinterpret_cast<unsigned short*>(sm + TrainSmem::XT + kmaj(6, r, kRows)) = one;
-        *reinterpret_cast<unsigned short*>(sm + TrainSmem::Bt + kmaj(128, r, kRows)) = one;
-    }
-    if (r == 0) mbar_init(s0 + TrainSmem::Bar);
-    if ((r >> 5) == 0) tmem_alloc(s0 + TrainSmem::Slot, kTrainCols);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tbase = *reinterpret_cast<volatile uint32_t*>(sm + TrainSmem::Slot);
-    const uint32_t t_row = tbase + ((uint32_t)((r >> 5) * 32) << 16);
-    const uint32_t bar = s0 + TrainSmem::Bar;
-    uint32_t phase = 0u;
-    bool ok = true;
-    int tiles_done = 0;
-    double loss_acc = 0.0;
-    const long long end = min(first + rows, n);
-    for (long long tile = blockIdx.x; first + tile * kRows < end && ok; tile += gridDim.x) {
-        const long long row = first + tile * kRows + r;
-        const bool valid = row < end;
-        // ---- inputs ----
-        float f[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-        if (valid) {
+            if (t > 0.0f) {
+                const float resp = expf(acc - L);
+                const float pi = expf(alpha - lse_a);
+                g[1] = pi - resp;
 #pragma unroll
-            for (int k = 0; k < 6; ++k) f[k] = __ldg(x + 6 * row + k);
-        }
-        store_input_row(sm + TrainSmem::X, r, f);
-#pragma unroll
-        for (int k = 0; k < 6; ++k)
-            *reinterpret_cast<unsigned short*>(sm + TrainSmem::XT + kmaj(k, r, kRows)) = bf16_bits(f[k]);
-        uint32_t m1[4] = {0u, 0u, 0u, 0u}, m2[4] = {0u, 0u, 0u, 0u};
-        // ---- layer 1 ----
-        publish();
-        if (r == 0) {
-            tc_fence_after();
-            mma_tile(tbase, s0 + TrainSmem::X, s0 + TrainSmem::Img + kImgW1, kInPad, kH, false);
-            umma_commit(bar);
-        }
-        if (!(ok = complete(bar, phase))) break;
-        hidden_epilogue_train(t_row, net.params + ob1, sm + TrainSmem::A, sm + TrainSmem::Bt, r, m1);
-        // ---- layer 2 ----
-        publish();
-        if (r == 0) {
-            tc_fence_after();
-            mma_tile(tbase + 128u, s0 + TrainSmem::A, s0 + TrainSmem::Img + kImgW2, kH, kH, false);
-            umma_commit(bar);
-        }
-        if (!(ok = complete(bar, phase))) break;
-        hidden_epilogue_train(t_row + 128u, net.params + ob2, sm + TrainSmem::A, sm + TrainSmem::C, r, m2);
-        // ---- output layer ----
-        publish();
-        if (r == 0) {
-            tc_fence_after();
-            mma_tile(tbase, s0 + TrainSmem::A, s0 + TrainSmem::Img + kImgW3, kH, kOutPad, false);
-            umma_commit(bar);
-        }
-        if (!(ok = complete(bar, phase))) break;
-        float zz[kOutPad], g[kOutPad];
-        output_epilogue(t_row, s_b3, zz);
-        float lrow = 0.0f;
-        if (valid) {
-            lrow = row_loss_grad(zz, label[row] > 0 ? 1.0f : 0.0f, yt + 5 * row, g);
-#pragma unroll
-            for (int j = 0; j < kOutPad; ++j) g[j] *= inv_rows;
-        } else {
-#pragma unroll
-            for (int j = 0; j < kOutPad; ++j) g[j] = 0.0f;
-        }
-        loss_acc += (double)lrow;
-        // dz: K-major [128 x 48] and transposed [48 x 128]; b3 gradient by warp sums
-#pragma unroll
-        for (int c0 = 0; c0 < kOutPad; c0 += 8) {
-            uint32_t w[4];
-#pragma unroll
-            for (int j = 0; j < 8; j += 2) w[j >> 1] = pack_bf16(g[c0 + j], g[c0 + j + 1]);
-            *reinterpret_cast<uint4*>(sm + TrainSmem::DZ + kmaj(r, c0, kOutPad)) = make_uint4(w[0], w[1], w[2], w[3]);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (c0 + j < kOut) {
-                    const unsigned short b = (unsigned short)((w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu);
-                    *reinterpret_cast<unsigned short*>(sm + TrainSmem::DZT + kmaj(c0 + j, r, kRows)) = b;
+                for (int j = 0; j < kDY; ++j) {
+                    const float s = zv[7 + j];
+                    const float inv2 = expf(-2.0f * s);
+                    const float diff = y[j] - zv[2 + j];
+                    g[2 + j] = -resp * diff * inv2;
+                    g[7 + j] = -resp * (diff * diff * inv2 - 1.0f);
                 }
             }
+#pragma unroll
+            for (int j = 0; j < 12; ++j) g[j] *= inv_rows;
         }
-#pragma unroll 1
-        for (int j = 0; j < kOut; ++j) {
-            const float s = warp_sum(g[j]);
-            if (lane == 0 && s != 0.0f) atomicAdd(s_db3 + j, s);
+        // dz [128 x 48] in the outputs' order, and b3's gradient by warp sums
+        const int col[12] = {0,          1 + cg,          5 + 5 * cg,      6 + 5 * cg,      7 + 5 * cg,      8 + 5 * cg,
+                             9 + 5 * cg, 25 + 5 * cg, 26 + 5 * cg, 27 + 5 * cg, 28 + 5 * cg, 29 + 5 * cg};
+#pragma unroll
+        for (int j = 0; j < 12; ++j) {
+            if (j == 0 && cg != 0) continue;
+            *reinterpret_cast<unsigned short*>(sm + S::DZ + kmaj(r, col[j], kOutPad)) = bf16_bits(g[j]);
         }
         // ---- dh2 = dz W3 and dW3^T += h2^T dz ----
         publish();
-        if (r == 0) {
+        if (threadIdx.x == 0) {
             tc_fence_after();
-            mma_tile(tbase, s0 + TrainSmem::DZ, s0 + TrainSmem::Img + kImgW3T, kOutPad, kH, false);
-            mma_tile(tbase + kColW3T, s0 + TrainSmem::C, s0 + TrainSmem::DZT, kRows, kOutPad, tiles_done > 0);
+            mma_operands(tbase, dzK, w3M, kOutPad, kH, false);
+            mma_operands(tbase + kColW3T, h2M, dzM, kRows, kOutPad, tiles_done > 0);
             umma_commit(bar);
         }
-        if (!(ok = complete(bar, phase))) break;
-        // ---- da2 = dh2 * relu'(a2): K-major into A, transposed into C ----
-        tmem_cols_pipelined(t_row, kH, [&](const uint32_t (&v)[16], int c0) {
-            const uint32_t mb = m2[c0 >> 5] >> (c0 & 31);
-            uint32_t w[8];
 #pragma unroll
-            for (int j = 0; j < 16; j += 2) {
-                const float a0 = ((mb >> j) & 1u) ? __uint_as_float(v[j]) : 0.0f;
-                const float a1 = ((mb >> (j + 1)) & 1u) ? __uint_as_float(v[j + 1]) : 0.0f;
-                w[j >> 1] = pack_bf16(a0, a1);
-                *reinterpret_cast<unsigned short*>(sm + TrainSmem::C + kmaj(c0 + j, r, kRows)) =
-                    (unsigned short)(w[j >> 1] & 0xFFFFu);
-                *reinterpret_cast<unsigned short*>(sm + TrainSmem::C + kmaj(c0 + j + 1, r, kRows)) =
-                    (unsigned short)(w[j >> 1] >> 16);
-            }
-            *reinterpret_cast<uint4*>(sm + TrainSmem::A + kmaj(r, c0, kH)) = make_uint4(w[0], w[1], w[2], w[3]);
-            *reinterpret_cast<uint4*>(sm + TrainSmem::A + kmaj(r, c0 + 8, kH)) = make_uint4(w[4], w[5], w[6], w[7]);
-        });
+        for (int j = 0; j < 12; ++j) {              // meanwhile: the rows' sums
+            const float sum = warp_sum(g[j]);
+            if (lane == 0 && (j > 0 || cg == 0)) s_red[kOutPad * q + col[j]] = sum;
+        }
+        ok = step() && ok;
+        // ---- da2 = dh2 * relu'(a2), over h2 ----
+        masked_epilogue(t_row, m2, sm + S::H2, r, c0);
         // ---- dh1 = da2 W2 and [dW2 | db2] += da2^T [h1 | 1] ----
         publish();
-        if (r == 0) {
+        if (threadIdx.x == 0) {
             tc_fence_after();
-            mma_tile(tbase + 128u, s0 + TrainSmem::A, s0 + TrainSmem::Img + kImgW2T, kH, kH, false);
-            mma_tile(tbase + kColW2, s0 + TrainSmem::C, s0 + TrainSmem::Bt, kRows, 144, tiles_done > 0);
+            mma_operands(tbase + 128u, h2K, w2M, kH, kH, false);
+            mma_operands(tbase + kColW2, h2M, h1M, kRows, kH1Cols, tiles_done > 0);
             umma_commit(bar);
         }
-        if (!(ok = complete(bar, phase))) break;
-        // ---- da1 = dh1 * relu'(a1), transposed into C ----
-        tmem_cols_pipelined(t_row + 128u, kH, [&](const uint32_t (&v)[16], int c0) {
-            const uint32_t mb = m1[c0 >> 5] >> (c0 & 31);
+        if (threadIdx.x < kOut) {
+            float d = s_db3[threadIdx.x];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float a = ((mb >> j) & 1u) ? __uint_as_float(v[j]) : 0.0f;
-                *reinterpret_cast<unsigned short*>(sm + TrainSmem::C + kmaj(c0 + j, r, kRows)) = bf16_bits(a);
-            }
-        });
+            for (int k = 0; k < 4; ++k) d += s_red[kOutPad * k + threadIdx.x];
+            s_db3[threadIdx.x] = d;
+        }
+        ok = step() && ok;
+        // ---- da1 = dh1 * relu'(a1), over da2 ----
+        masked_epilogue(t_row + 128u, m1, sm + S::H2, r, c0);
         // ---- [dW1 | db1] += da1^T [x | 1] ----
         publish();
-        if (r == 0) {
+        if (threadIdx.x == 0) {
             tc_fence_after();
-            mma_tile(tbase + kColW1, s0 + TrainSmem::C, s0 + TrainSmem::XT, kRows, kInPad, tiles_done > 0);
+            mma_operands(tbase + kColW1, h2M, xM, kRows, kInPad, tiles_done > 0);
             umma_commit(bar);
         }
-        if (!(ok = complete(bar, phase))) break;
+        ok = step() && ok;
         ++tiles_done;
     }
     // ---- loss and the accumulated weight gradients ----
-    const float ls = warp_sum((float)loss_acc);
-    if (lane == 0 && ls != 0.0f) atomicAdd(net.loss, (double)ls);
+    if (cg == 0) {
+        const float ls = warp_sum((float)loss_acc);
+        if (lane == 0 && ls != 0.0f) atomicAdd(net.loss, (double)ls);
+    }
     // the CTA's partial gradient, every parameter written once (plain stores;
     // the Adam step sums the CTAs' partials: no contended atomics)
     float* part = net.gpart + (long long)blockIdx.x * kNParams;
-    const bool have = ok && tiles_done > 0;
-    __syncthreads();                                // s_db3 complete
+    const bool have = __syncthreads_and(ok) && tiles_done > 0;
     {
         const int h = r;
-#pragma unroll 1
-        for (int c0 = 0; c0 < 144; c0 += 16) {
-            float v[16];
-            if (have) tmem_ld16(t_row + kColW2 + (uint32_t)c0, v);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int i = c0 + j;
-                const float gv = have ? v[j] : 0.0f;
-                if (i < kH) part[oW2 + h * kH + i] = gv;
-                else if (i == kH) part[ob2 + h] = gv;
+        store_partial<32>(t_row + kColW2 + (uint32_t)c0, have, part + oW2 + h * kH + c0);
+        if (cg == 0) store_partial<1>(t_row + kColW2 + kH, have, part + ob2 + h);
+        if (cg < 3) {
+            uint32_t v[16];
+            if (have) {
+                tmem_ld16_async(t_row + kColW3T + (uint32_t)(16 * cg), v);
+                tmem_wait16(v);
             }
-        }
-#pragma unroll 1
-        for (int c0 = 0; c0 < kOutPad; c0 += 16) {
-            float v[16];
-            if (have) tmem_ld16(t_row + kColW3T + (uint32_t)c0, v);
 #pragma unroll
             for (int j = 0; j < 16; ++j)
-                if (c0 + j < kOut) part[oW3 + (c0 + j) * kH + h] = have ? v[j] : 0.0f;
-        }
-        {
-            float v[16];
-            if (have) tmem_ld16(t_row + kColW1, v);
+                if (16 * cg + j < kOut) part[oW3 + (16 * cg + j) * kH + h] = have ? __uint_as_float(v[j]) : 0.0f;
+        } else {
+            uint32_t v[16];
+            if (have) {
+                tmem_ld16_async(t_row + kColW1, v);
+                tmem_wait16(v);
+            }
 #pragma unroll
-            for (int j = 0; j < kIn; ++j) part[oW1 + h * kIn + j] = have ? v[j] : 0.0f;
-            part[ob1 + h] = have ? v[kIn] : 0.0f;
+            for (int j = 0; j < kIn; ++j) part[oW1 + h * kIn + j] = have ? __uint_as_float(v[j]) : 0.0f;
+            part[ob1 + h] = have ? __uint_as_float(v[kIn]) : 0.0f;
         }
-        if (r < kOut) part[ob3 + r] = have ? s_db3[r] : 0.0f;
+        if (threadIdx.x < kOut) part[ob3 + threadIdx.x] = have ? s_db3[threadIdx.x] : 0.0f;
     }
-    if (!ok) {
-        if (r == 0) atomicOr(net.status, 1);
+    if (!ok) {                                      // a wait failed in this thread
+        atomicOr(net.status, 1);
         (void)mbar_wait(bar, phase);
     }
     tc_fence_before();
     __syncthreads();
-    if ((r >> 5) == 0) {
+    if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tbase, kTrainCols);
     }
@@ -1062,11 +1149,10 @@ __device__ __forceinline__ void write_images(unsigned char* img, int k, float w)
     } else if (k >= oW2 && k < ob2) {
         const int h = (k - oW2) / kH, i = (k - oW2) % kH;
         *reinterpret_cast<unsigned short*>(img + kImgW2 + kmaj(h, i, kH)) = b;
-        *reinterpret_cast<unsigned short*>(img + kImgW2T + kmaj(i, h, kH)) = b;
     } else if (k >= oW3 && k < ob3) {
         const int o = (k - oW3) / kH, h = (k - oW3) % kH;
         *reinterpret_cast<unsigned short*>(img + kImgW3 + kmaj(o, h, kH)) = b;
-        *reinterpret_cast<unsigned short*>(img + kImgW3T + kmaj(h, o, kOutPad)) = b;
+        *reinterpret_cast<unsigned short*>(img + kImgW3P + kmaj(w3p_row(o), h, kH)) = b;
     }
 }
 
@@ -1076,13 +1162,22 @@ __global__ void k_sur_pack(const SurNet net)
     if (k < kNParams) write_images(net.img, k, net.params[k]);
 }
 
-// Adam (Kingma & Ba 2015): moments, bias corrections c1 = 1 / (1 - beta1^t),
-// c2 = 1 / (1 - beta2^t); the gradient is cleared for the next step.
-// Sum of the parts CTAs' partial gradients of parameter k (coalesced over k).
+// Sum of the parts CTAs' partial gradients of parameter k (coalesced over k),
+// in the CTAs' order; 16 loads in flight.
 __device__ __forceinline__ float summed_grad(const SurNet& net, int k, int parts)
 {
+    constexpr int kU = 16;
     float g = 0.0f;
-    for (int c = 0; c < parts; ++c) g += net.gpart[(long long)c * kNParams + k];
+    const float* p = net.gpart + k;
+    int c = 0;
+    for (; c + kU <= parts; c += kU) {
+        float v[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) v[u] = p[(long long)(c + u) * kNParams];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) g += v[u];
+    }
+    for (; c < parts; ++c) g += p[(long long)c * kNParams];
     return g;
 }
 
@@ -1092,6 +1187,8 @@ __global__ void k_sur_reduce(const SurNet net, int parts)
     if (k < kNParams) net.grad[k] = summed_grad(net, k, parts);
 }
 
+// Adam (Kingma & Ba 2015): moments, bias corrections c1 = 1 / (1 - beta1^t),
+// c2 = 1 / (1 - beta2^t).
 __global__ void k_sur_adam(const SurNet net, float lr, float c1, float c2, int parts)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1157,7 +1254,7 @@ cudaError_t launch_sur_train(const SurNet& net, const float* x, const float* y, 
     const long long tiles = (rows + kRows - 1) / kRows;
     if (tiles <= 0) return cudaSuccess;
     const int ctas = (int)std::min<long long>(tiles, std::min(grid, net.n_part_cap));
-    k_sur_train<<<ctas, kRows, TrainSmem::Bytes, s>>>(net, x, y, label, first, rows, n, inv_rows);
+    k_sur_train<<<ctas, kTrainThreads, TrainSmem::Bytes, s>>>(net, x, y, label, first, rows, n, inv_rows);
     *parts = ctas;
     return cudaGetLastError();
 }

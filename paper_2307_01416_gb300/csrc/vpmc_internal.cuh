@@ -115,13 +115,13 @@ constexpr int oW1 = 0, ob1 = oW1 + kH * kIn, oW2 = ob1 + kH, ob2 = oW2 + kH * kH
 constexpr int kNParams = ob3 + kOut;
 // BF16 operand images in the canonical no-swizzle K-major layout of the
 // tensor-core instructions (byte offsets): W1 [128 x 16], W2 [128 x 128],
-// W3 [48 x 128], and the transposes W2^T [128 x 128], W3^T [128 x 48].
+// W3 [48 x 128], and W3's rows in the training kernel's order [64 x 128].
+constexpr int kOutP = 64;
 constexpr int kImgW1 = 0;
 constexpr int kImgW2 = kImgW1 + kH * kInPad * 2;
 constexpr int kImgW3 = kImgW2 + kH * kH * 2;
-constexpr int kImgW2T = kImgW3 + kOutPad * kH * 2;
-constexpr int kImgW3T = kImgW2T + kH * kH * 2;
-constexpr int kImgBytes = kImgW3T + kH * kOutPad * 2;
+constexpr int kImgW3P = kImgW3 + kOutPad * kH * 2;
+constexpr int kImgBytes = kImgW3P + kOutP * kH * 2;
 // Input and target scales, training domain.
 constexpr float kDCap = 12.0f;       // mm: edge distance clip
 constexpr float kELo = 40.0f, kEHi = 230.0f;
