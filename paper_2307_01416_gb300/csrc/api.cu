@@ -1830,8 +1830,6 @@ struct OptInputs {
     std::vector<const float*> val;
     long long n_rows = 0;
     int n_cols = 0;
-    long long n_target = 0, n_ring = 0;
-    std::vector<unsigned char> cls;         // host copy of the voxel classes
 };
 
 vpmc_status check_opt_inputs(const vpmc_csr* mats, int n_scen, const uint8_t* cls, OptInputs* in)
@@ -1851,14 +1849,6 @@ vpmc_status check_opt_inputs(const vpmc_csr* mats, int n_scen, const uint8_t* cl
     if (in->n_rows <= 0 || mats[0].n_cols <= 0) return fail(VPMC_ERR_ARG, "empty matrices");
     if (mats[0].n_cols > 28000) return fail(VPMC_ERR_ARG, "%lld columns: at most 28,000", (long long)mats[0].n_cols);
     if (in->n_rows > INT32_MAX) return fail(VPMC_ERR_ARG, "more than 2^31 - 1 rows");
-    std::vector<unsigned char>& h = in->cls;
-    h.resize((size_t)in->n_rows);
-    if (cudaMemcpy(h.data(), cls, h.size(), cudaMemcpyDeviceToHost) != cudaSuccess)
-        return fail(VPMC_ERR_CUDA, "reading the voxel classes: %s", cudaGetErrorString(cudaGetLastError()));
-    for (unsigned char c : h) {
-        in->n_target += c == 1;
-        in->n_ring += c == 2;
-    }
     return VPMC_OK;
 }
 
@@ -1886,30 +1876,35 @@ vpmc_status vpmc_robust_optimize(const vpmc_csr* mats, int n_scen, const uint8_t
     OptInputs in;
     vpmc_status st = check_opt_inputs(mats, n_scen, voxel_class_dev, &in);
     if (st != VPMC_OK) return st;
-    if (in.n_target == 0) return fail(VPMC_ERR_ARG, "no target voxels (class 1)");
+    OptSpec spec;
+    ClassRows* rows = nullptr;
+    struct RowsFree {
+        ClassRows*& r;
+        ~RowsFree() { free_class_rows(r); }
+    } rows_free{rows};
+    CUDA_TRY(count_class_rows(voxel_class_dev, in.n_rows, (cudaStream_t)stream, &rows, &spec.n_target, &spec.n_ring));
+    if (spec.n_target == 0) return fail(VPMC_ERR_ARG, "no target voxels (class 1)");
     std::vector<float> x0((size_t)in.n_cols);
-    CUDA_TRY(cudaMemcpy(x0.data(), x_dev, x0.size() * sizeof(float), cudaMemcpyDeviceToHost));
+    CUDA_TRY(cudaMemcpyAsync(x0.data(), x_dev, x0.size() * sizeof(float), cudaMemcpyDeviceToHost, (cudaStream_t)stream));
+    CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
     double mean = 0.0;
     for (float v : x0) {
         if (!(v >= 0.0f) || !std::isfinite(v)) return fail(VPMC_ERR_ARG, "initial weights must be finite and >= 0");
         mean += v;
     }
     mean /= (double)x0.size();
-    OptSpec spec;
     spec.dp = prm->prescription;
     spec.w_u = prm->w_under;
     spec.w_o = prm->w_over;
     spec.w_r = prm->w_ring;
     spec.over = prm->over_frac;
     spec.ring = prm->ring_frac;
-    spec.n_target = in.n_target;
-    spec.n_ring = in.n_ring;
     spec.step = (float)(prm->lr * (mean > 0.0 ? mean : 1.0));
     spec.eps = 1e-8f;
     spec.iterations = prm->iterations;
     float t[2] = {0.0f, 0.0f};
     CUDA_TRY(run_robust_optimize(in.rp.data(), in.col.data(), in.val.data(), n_scen, in.n_rows, in.n_cols,
-                                 in.cls.data(), spec, x_dev, history, (cudaStream_t)stream, t, nullptr));
+                                 voxel_class_dev, *rows, spec, x_dev, history, (cudaStream_t)stream, t, nullptr));
     if (ms) {
         ms[0] = t[0];
         ms[1] = t[1];

@@ -316,7 +316,7 @@ size_t sur_train_smem_bytes();
 
 // Robust spot-weight optimisation (optimize.cu).  Matrices: n_scen CSR of
 // n_rows x n_cols (device pointers); cls: uint8 voxel classes (1 target,
-// 2 ring); x: device weights, optimised in place.
+// 2 ring; device); x: device weights, optimised in place.
 struct OptSpec {
     float dp, w_u, w_o, w_r, over, ring;    // prescription, weights, over- and ring-dose fractions
     long long n_target, n_ring;
@@ -327,9 +327,16 @@ struct OptSetupInfo {
     long long n_tr, nnz_tr;                 // target + ring rows; their entries over all scenarios
     long long compact_entries;              // padded size of the compact CSR
 };
+// Counts the target and ring voxels of cls (device), keeping on the device
+// what run_robust_optimize needs of them; *rows is always to be freed.
+struct ClassRows;
+cudaError_t count_class_rows(const unsigned char* cls, long long n_rows, cudaStream_t st, ClassRows** rows,
+                             long long* n_target, long long* n_ring);
+void free_class_rows(ClassRows* rows);
 cudaError_t run_robust_optimize(const long long* const* rp, const int* const* col, const float* const* val, int n_scen,
-                                long long n_rows, int n_cols, const unsigned char* cls_host, const OptSpec& spec,
-                                float* x, float* hist_host, cudaStream_t st, float* ms_out, OptSetupInfo* info);
+                                long long n_rows, int n_cols, const unsigned char* cls, const ClassRows& rows,
+                                const OptSpec& spec, float* x, float* hist_host, cudaStream_t st, float* ms_out,
+                                OptSetupInfo* info);
 cudaError_t run_weights_dose(const long long* rp, const int* col, const float* val, long long n_rows, int n_cols,
                              const float* x, float* dose, cudaStream_t st, int num_sms);
 cudaError_t run_target_indices(const long long* const* rp, const int* const* col, const float* const* val, int n_scen,
