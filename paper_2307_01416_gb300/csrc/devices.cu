@@ -12,7 +12,8 @@
 // decides opening -> straight flight, or brass -> condensed-history step with
 // brass physics); k_patient (patient.cu) transports it through the voxelised
 // patient.  Each kernel is compiled twice: with the physics switches read
-// from the launch, and with full physics known at compile time.
+// from the launch, and with full physics and the 32-bit fixed-point conversion
+// known at compile time (the 64-bit one takes the FP64 pipe).
 #include "transport_common.cuh"
 
 namespace vpmc {
@@ -52,6 +53,7 @@ __device__ __forceinline__ bool local_point_in_polygon(uint32_t local, float x, 
     bool c = (local >> 31) != 0u;
     int i = (int)(local & 0xffffu);
     float2 pj = poly[off + (i == 0 ? n - 1 : i - 1)];
+#pragma unroll 1
     for (int k = (int)(local >> 16) & 0x7fff; k > 0; --k) {
         const float2 pi = poly[off + i];
         c ^= edge_crosses(x, y, pi, pj);
@@ -73,6 +75,7 @@ __device__ __forceinline__ bool coop_point_in_polygon(bool need, float x, float 
         const float qx = __shfl_sync(kFull, x, src), qy = __shfl_sync(kFull, y, src);
         const int qo = __shfl_sync(kFull, off, src), qn = __shfl_sync(kFull, n, src);
         bool c = false;
+#pragma unroll 1
         for (int i = lane; i < qn; i += 32) {
             const float2 pi = poly[qo + i];
             const float2 pj = poly[qo + (i == 0 ? qn - 1 : i - 1)];
@@ -145,6 +148,7 @@ __device__ __forceinline__ float coop_wall_distance(bool need, float x, float y,
         const float qx = __shfl_sync(kFull, x, src), qy = __shfl_sync(kFull, y, src);
         const int qo = __shfl_sync(kFull, off, src), qn = __shfl_sync(kFull, n, src);
         float best = __int_as_float(0x7f800000);
+#pragma unroll 1
         for (int i = lane; i < qn; i += 32) {
             best = fminf(best, edge_distance2(qx, qy, poly, qo, qn, i));
         }
@@ -176,6 +180,7 @@ __device__ __forceinline__ float4 coop_nearest_edge(bool need, float x, float y,
         const int qo = __shfl_sync(kFull, off, src), qn = __shfl_sync(kFull, n, src);
         float best = __int_as_float(0x7f800000), bt = 0.0f;
         int bi = 0x7fffffff;
+#pragma unroll 1
         for (int i = lane; i < qn; i += 32) {
             const float2 a = poly[qo + i];
             const float2 b = poly[qo + (i + 1 < qn ? i + 1 : 0)];
@@ -285,11 +290,14 @@ __global__ void __launch_bounds__(768, 1) k_source_rs(const TransportParams P)
     {
         float2* R = reinterpret_cast<float2*>(smem + SourceSmem::R);
         float2* Et = reinterpret_cast<float2*>(smem + SourceSmem::Einv);
+#pragma unroll 1
         for (int i = threadIdx.x; i < kNEPad; i += blockDim.x) R[i] = P.tables->R[kPMMA][i];
+#pragma unroll 1
         for (int i = threadIdx.x; i < kNR; i += blockDim.x) Et[i] = P.tables->Einv[kPMMA][i];
         MatConst* mt = reinterpret_cast<MatConst*>(smem + SourceSmem::Mat);
         if (threadIdx.x < kNMat) mt[threadIdx.x] = P.tables->mat[threadIdx.x];
         DevBeam* bm = reinterpret_cast<DevBeam*>(smem + SourceSmem::Beams);
+#pragma unroll 1
         for (int i = threadIdx.x; i < P.n_beams; i += blockDim.x) bm[i] = P.beams[i];
     }
     __syncthreads();
@@ -388,7 +396,7 @@ __global__ void __launch_bounds__(768, 1) k_source_rs(const TransportParams P)
                 StepResult o;
                 ch_step<kAllPhysics>(pmma, s_geom, L, P, draw, o);
                 acc_steps += 1;
-                const unsigned long long qs = to_fixed(o.dE, P.fscale, P.fx32);
+                const unsigned long long qs = to_fixed(o.dE, P.fscale, kAllPhysics || P.fx32);
                 acc_rs += qs;
                 if (o.killed) {
                     if (o.killed == 2) acc_nuc += qs;
@@ -400,7 +408,7 @@ __global__ void __launch_bounds__(768, 1) k_source_rs(const TransportParams P)
                 }
             }
             if (fate >= 0) {
-                if (fate == kLeak || fate == kErr) acc_leak += to_fixed(L.E, P.fscale, P.fx32);
+                if (fate == kLeak || fate == kErr) acc_leak += to_fixed(L.E, P.fscale, kAllPhysics || P.fx32);
                 if (fate == kErr) { acc_err += 1; atomicOr(P.status, 1); }
                 if (P.records && L.g < P.rec_cap) {
                     float pos[3];
@@ -461,10 +469,15 @@ __global__ void __launch_bounds__(768, 1) k_source_rs(const TransportParams P)
 // history.  Lanes take new histories eight at a time (four or eight: the same;
 // one: 7 to 17 % slower), in blocks of 24 warps at 80 registers (640 threads
 // at 96: 0.5 to 2 % slower behind an aperture, the same on tracks).
-// 4e6 histories behind range shifter and aperture: 8.4 ms, now 6.9 ms; 2e6
-// training tracks 16.0 -> 8.2 ms; histories at the rim of a 256-gon of 10 mm,
-// 4.1 ms, as before.  Letting the histories that start in the opening fly
-// during the refill (they mostly pass straight through) lost 20 to 25 %.
+// The loops over edges, scenarios and staged tables are not unrolled: 70 KB of
+// code for 24 warps at as many places spent a third of the time on instruction
+// fetches (45 KB now; the wall-hit loop stays as it was compiled, the rounding
+// of its products with it).
+// 4e6 histories behind range shifter and aperture: 8.4 ms at first, 6.9 ms
+// with the raster's edges, 5.4 ms without the unrolling; 2e6 training tracks
+// 16.0, 8.2, 6.1 ms; histories at the rim of a 256-gon of 10 mm 4.1, 4.1, 3.1
+// ms.  Letting the histories that start in the opening fly during the refill
+// (they mostly pass straight through) lost 20 to 25 %.
 // kMode bit 0: brass entries in the surrogate's domain become queries;
 // bit 1: training tracks (histories start on the aperture entrance plane and
 // record the surrogate's inputs and targets).
@@ -479,15 +492,20 @@ __global__ void __launch_bounds__(768, 1) k_aperture(const TransportParams P)
         // brass rows of the tables, material constants, beams, scenarios, polygons
         float2* R = reinterpret_cast<float2*>(smem + ApertureSmem::R);
         float2* Et = reinterpret_cast<float2*>(smem + ApertureSmem::Einv);
+#pragma unroll 1
         for (int i = threadIdx.x; i < kNEPad; i += blockDim.x) R[i] = P.tables->R[kBrass][i];
+#pragma unroll 1
         for (int i = threadIdx.x; i < kNR; i += blockDim.x) Et[i] = P.tables->Einv[kBrass][i];
         MatConst* mt = reinterpret_cast<MatConst*>(smem + ApertureSmem::Mat);
         if (threadIdx.x < kNMat) mt[threadIdx.x] = P.tables->mat[threadIdx.x];
         DevBeam* bm = reinterpret_cast<DevBeam*>(smem + ApertureSmem::Beams);
+#pragma unroll 1
         for (int i = threadIdx.x; i < P.n_beams; i += blockDim.x) bm[i] = P.beams[i];
         DevScen* sc = reinterpret_cast<DevScen*>(smem + ApertureSmem::Scens);
+#pragma unroll 1
         for (int i = threadIdx.x; i < P.n_scen; i += blockDim.x) sc[i] = P.scens[i];
         float2* pl = reinterpret_cast<float2*>(smem + ApertureSmem::Poly);
+#pragma unroll 1
         for (int i = threadIdx.x; i < P.n_poly; i += blockDim.x) pl[i] = P.poly[i];
     }
     __syncthreads();
@@ -539,6 +557,7 @@ __global__ void __launch_bounds__(768, 1) k_aperture(const TransportParams P)
                 r.E = L.E;
                 r.nlam = L.nlam;
                 r.step = L.step;
+#pragma unroll 1
                 for (int s = 0; s < P.n_rep; ++s) {
                     bev_to_patient(B, scens[scen0 + s], L.p, r.p);
                     r.item = L.item + s * P.rep_items;
@@ -822,7 +841,7 @@ __global__ void __launch_bounds__(768, 1) k_aperture(const TransportParams P)
                     if (need_dist) absorb = rmax < dw;
                     else if (kSur && reaches) absorb = false;
                     if (absorb) {
-                        acc_ap += to_fixed(L.E, P.fscale, P.fx32);
+                        acc_ap += to_fixed(L.E, P.fscale, kAllPhysics || P.fx32);
                         L.E = 0.0f;
                         fate = kAbsAp;
                     } else {
@@ -835,7 +854,7 @@ __global__ void __launch_bounds__(768, 1) k_aperture(const TransportParams P)
                 StepResult o;
                 ch_step<kAllPhysics>(m, s_geom, L, P, draw, o);
                 acc_steps += 1;
-                const unsigned long long qs = to_fixed(o.dE, P.fscale, P.fx32);
+                const unsigned long long qs = to_fixed(o.dE, P.fscale, kAllPhysics || P.fx32);
                 acc_ap += qs;
                 if (o.killed) {
                     if (o.killed == 2) acc_nuc += qs;
@@ -865,7 +884,7 @@ __global__ void __launch_bounds__(768, 1) k_aperture(const TransportParams P)
             }
             if (fate >= 0) {
                 // the single place where a history ends in this kernel
-                if (fate == kLeak || fate == kErr) acc_leak += to_fixed(L.E, P.fscale, P.fx32);
+                if (fate == kLeak || fate == kErr) acc_leak += to_fixed(L.E, P.fscale, kAllPhysics || P.fx32);
                 if (fate == kErr) { acc_err += 1; atomicOr(P.status, 1); }
                 if (P.records && L.g < P.rec_cap) {
                     float pos[3];
@@ -929,7 +948,7 @@ static cudaError_t launch_aperture_variant(const TransportParams& p, int grid, i
 template <int kMode>
 static cudaError_t launch_aperture_mode(const TransportParams& p, int grid, int block, cudaStream_t s)
 {
-    if (p.mcs && p.straggling && p.nuclear) return launch_aperture_variant<kMode, true>(p, grid, block, s);
+    if (p.mcs && p.straggling && p.nuclear && p.fx32) return launch_aperture_variant<kMode, true>(p, grid, block, s);
     return launch_aperture_variant<kMode, false>(p, grid, block, s);
 }
 
@@ -953,7 +972,7 @@ cudaError_t launch_devices(const TransportParams& p, int grid, int block, cudaSt
     if (!p.track_mode) {
         cudaError_t e = cudaMemsetAsync(p.mid_count, 0, sizeof(unsigned long long), s);
         if (e != cudaSuccess) return e;
-        e = (p.mcs && p.straggling && p.nuclear) ? launch_source_rs<true>(p, grid, s) : launch_source_rs<false>(p, grid, s);
+        e = (p.mcs && p.straggling && p.nuclear && p.fx32) ? launch_source_rs<true>(p, grid, s) : launch_source_rs<false>(p, grid, s);
         if (e != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(p.counter, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
     }
