@@ -1561,10 +1561,12 @@ vpmc_status reset_optimizer(vpmc_ctx* c)
     return VPMC_OK;
 }
 
+// Waits for the stream's work and reads the tensor-core status word behind it.
 vpmc_status surrogate_status(vpmc_ctx* c)
 {
     int ss = 0;
-    CUDA_TRY(cudaMemcpy(&ss, c->sur.status, sizeof ss, cudaMemcpyDeviceToHost));
+    CUDA_TRY(cudaMemcpyAsync(&ss, c->sur.status, sizeof ss, cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
     if (ss) return fail(VPMC_ERR_TIMEOUT, "surrogate: a tensor-core wait timed out");
     return VPMC_OK;
 }
@@ -1642,7 +1644,6 @@ vpmc_status vpmc_surrogate_forward(vpmc_ctx* c, const float* feat_dev, int64_t n
     if (!c->sur_ready) return fail(VPMC_ERR_STATE, "no surrogate weights");
     CUDA_TRY(launch_sur_forward(c->sur, feat_dev, n, z_dev, c->num_sms, c->stream));
     ++c->launches;
-    CUDA_TRY(cudaStreamSynchronize(c->stream));
     return surrogate_status(c);
 }
 
@@ -1665,9 +1666,9 @@ vpmc_status vpmc_surrogate_gradient(vpmc_ctx* c, const float* feat_dev, const fl
     CUDA_TRY(cudaMemsetAsync(c->sur.grad, 0, sur::kNParams * sizeof(float), c->stream));
     double h[2] = {0.0, 0.0};
     CUDA_TRY(cudaMemcpyAsync(h, c->sur.loss, sizeof h, cudaMemcpyDeviceToHost, c->stream));
-    CUDA_TRY(cudaStreamSynchronize(c->stream));
+    const vpmc_status st = surrogate_status(c);
     if (loss) *loss = h[0] / (double)n;
-    return surrogate_status(c);
+    return st;
 }
 
 vpmc_status vpmc_surrogate_train(vpmc_ctx* c, const float* feat_dev, const float* target_dev, const int32_t* label_dev,
@@ -1704,9 +1705,8 @@ vpmc_status vpmc_surrogate_train(vpmc_ctx* c, const float* feat_dev, const float
         }
         double h[2] = {0.0, 0.0};
         CUDA_TRY(cudaMemcpyAsync(h, c->sur.loss, sizeof h, cudaMemcpyDeviceToHost, c->stream));
-        CUDA_TRY(cudaStreamSynchronize(c->stream));
-        if (epoch_loss) epoch_loss[e] = (float)(h[0] / (double)n);
         vpmc_status st = surrogate_status(c);
+        if (epoch_loss) epoch_loss[e] = (float)(h[0] / (double)n);
         if (st != VPMC_OK) return st;
         if (!std::isfinite(h[0]))
             return fail(VPMC_ERR_STATE, "training diverged in epoch %d (non-finite loss); lower lr or fewer steps", e);

@@ -578,22 +578,6 @@ struct Arena {
     T* at(size_t offset) const { return reinterpret_cast<T*>(base + offset); }
 };
 
-template <class... P, class... A>
-static cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A... args)
-{
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c{};
-    c.gridDim = grid;
-    c.blockDim = dim3(block);
-    c.dynamicSmemBytes = smem;
-    c.stream = st;
-    c.attrs = &at;
-    c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
-}
-
 // Counts the target and ring voxels (classes 1 and 2); *ws keeps the device
 // arrays for run_robust_optimize and is freed by free_class_rows.
 struct ClassRows {

@@ -270,6 +270,25 @@ static_assert(ApertureSmem::Bytes <= 227 * 1024, "aperture kernel shared memory"
 static_assert(PatientSmem::Bytes <= 227 * 1024, "patient kernel shared memory");
 static_assert(kPatientMaxBlock % 32 == 0, "whole warps");
 
+// Launches kernel with programmatic serialisation: it may start once every
+// block of the stream's last kernel has called launch_dependents (or ended),
+// and waits for that kernel's results itself (griddepcontrol.wait).
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // Host-side launchers (transport.cu, finalize.cu).
 // Transport of histories [p.hist_begin, p.total): the beam-line kernels
 // (source and range shifter, then the aperture: launch_devices, which resets
