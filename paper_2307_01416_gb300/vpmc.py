@@ -186,8 +186,23 @@ def make_opts(o: W.Options, aggregate: int = -1, block_size: int = 0, chunk: int
     return v
 
 
+_SPOT_FIELDS = (("beam", "beam"), ("energy_mev", "energy"), ("x_mm", "x"), ("y_mm", "y"), ("sigma_mm", "sigma"),
+                ("div_mrad", "div_mrad"), ("n_hist", "n_hist"), ("weight", "weight"))
+
+
 def spot_array(spots: np.ndarray):
-    arr = (vpmc_spot * max(len(spots), 1))()
+    """The spots as an array of vpmc_spot.  A structured array is copied field
+    by field (one numpy copy each: 3 us a spot otherwise, 16 ms of a 5,220-spot
+    dose call); any other sequence of records row by row."""
+    n = len(spots)
+    kinds = spots.dtype.fields if n and isinstance(spots, np.ndarray) and spots.ndim == 1 else None
+    if kinds and all(name in kinds and kinds[name][0].kind in ("iu" if field in ("beam", "n_hist") else "iuf")
+                     for field, name in _SPOT_FIELDS):
+        rows = np.zeros(n, dtype=np.dtype(vpmc_spot))
+        for field, name in _SPOT_FIELDS:
+            rows[field] = spots[name]
+        return (vpmc_spot * n).from_buffer(rows)
+    arr = (vpmc_spot * max(n, 1))()
     for i, s in enumerate(spots):
         arr[i] = vpmc_spot(int(s["beam"]), float(s["energy"]), float(s["x"]), float(s["y"]), float(s["sigma"]),
                            float(s["div_mrad"]), int(s["n_hist"]), float(s["weight"]))
