@@ -222,8 +222,9 @@ __global__ void __launch_bounds__(kPatientMaxBlock, 1) k_patient(const Transport
                 for (int k = 0; k < 3; ++k) {
                     const bool nested = (kNest >> k) & 1;
                     const float fc = (float)L.ic[k];
-                    f0[k] = P.ctg.lo[k] + fc * P.ctg.d[k];
-                    f1[k] = P.ctg.lo[k] + (fc + 1.0f) * P.ctg.d[k];
+                    const float2 ff = fma2(make_float2(fc, fc + 1.0f), both(P.ctg.d[k]), both(P.ctg.lo[k]));
+                    f0[k] = ff.x;
+                    f1[k] = ff.y;
                     if (!nested) {
                         const float fs = (float)L.is[k];
                         g0[k] = P.sg.lo[k] + fs * P.sg.d[k];
@@ -232,15 +233,14 @@ __global__ void __launch_bounds__(kPatientMaxBlock, 1) k_patient(const Transport
                     const float vlo = nested ? f0[k] : fmaxf(f0[k], g0[k]);
                     const float vhi = nested ? f1[k] : fminf(f1[k], g1[k]);
                     L.p[k] = fminf(fmaxf(L.p[k], vlo), vhi);
-                    dc[k] = ds[k] = __int_as_float(0x7f800000);
+                    // (a zero component: the face is chosen by its sign, so
+                    // that the quotient is +inf, or NaN on the face itself;
+                    // neither limits the step nor equals its length)
                     const float Dk = L.d[k];
-                    if (Dk != 0.0f) {
-                        const float inv = __fdividef(1.0f, Dk);
-                        const bool up = Dk > 0.0f;
-                        dc[k] = ((up ? f1[k] : f0[k]) - L.p[k]) * inv;
-                        if (nested) ds[k] = dc[k];
-                        else ds[k] = ((up ? g1[k] : g0[k]) - L.p[k]) * inv;
-                    }
+                    const float inv = __fdividef(1.0f, Dk);
+                    const bool up = __float_as_int(Dk) >= 0;
+                    dc[k] = ((up ? f1[k] : f0[k]) - L.p[k]) * inv;
+                    ds[k] = nested ? dc[k] : ((up ? g1[k] : g0[k]) - L.p[k]) * inv;
                     s_geom = fminf(s_geom, nested ? dc[k] : fminf(dc[k], ds[k]));
                     d_old[k] = Dk;
                 }
