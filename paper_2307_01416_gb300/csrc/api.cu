@@ -326,7 +326,7 @@ vpmc_status pending_status(vpmc_ctx* c)
     const bool sur = c->status_pending == 2;
     c->status_pending = 0;
     int status = 0, ss = 0;
-    CUDA_TRY(cudaMemcpyAsync(&status, c->d_status, sizeof status, cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(&status, &c->d_ctl->status, sizeof status, cudaMemcpyDeviceToHost, c->stream));
     if (sur && c->sur.status) CUDA_TRY(cudaMemcpyAsync(&ss, c->sur.status, sizeof ss, cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     if (status & 1) return fail(VPMC_ERR_TIMEOUT, "an earlier asynchronous call: histories reached the iteration cap");
@@ -348,6 +348,7 @@ TransportParams base_params(vpmc_ctx* c, const vpmc_opts& o)
     for (int k = 0; k < 3; ++k) p.nest_shift[k] = c->nest_shift[k];
     p.beams = c->d_beams;
     p.n_beams = kMaxBeams;
+    beam_flags(&p, c->beams, kMaxBeams);
     p.scens = c->d_scens;
     p.poly = c->d_poly;
     p.n_poly = c->n_poly;
@@ -358,9 +359,7 @@ TransportParams base_params(vpmc_ctx* c, const vpmc_opts& o)
     p.range_rejection = o.range_rejection;
     p.items = c->d_items;
     p.boxes = c->d_boxes;
-    p.counter = c->d_counter;
-    p.stats = c->d_stats;
-    p.status = c->d_status;
+    set_control(&p, c->d_ctl);
     p.key0 = (uint32_t)o.seed;
     p.key1_hi = (uint32_t)(o.seed >> 32);
     p.mcs = o.mcs;
@@ -373,10 +372,8 @@ TransportParams base_params(vpmc_ctx* c, const vpmc_opts& o)
     p.rec_cap = o.history_out ? o.history_cap : 0;
     p.phase = c->d_phase;
     p.phase_cap = c->phase_cap;
-    p.phase_count = c->d_phase_count;
     p.mid = c->d_mid;
     p.mid_cap = c->phase_cap;
-    p.mid_count = c->d_mid_count;
     p.poly_kappa = c->d_poly_kappa;
     p.surrogate = o.surrogate && c->sur_ready ? 1 : 0;
     p.n_rep = 1;                    // set by the influence-matrix path when scenarios share the beam line
@@ -386,9 +383,7 @@ TransportParams base_params(vpmc_ctx* c, const vpmc_opts& o)
 
 vpmc_status reset_counters(vpmc_ctx* c)
 {
-    CUDA_TRY(cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), c->stream));
-    CUDA_TRY(cudaMemsetAsync(c->d_stats, 0, sizeof(unsigned long long) * kNStats, c->stream));
-    CUDA_TRY(cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream));
+    CUDA_TRY(cudaMemsetAsync(c->d_ctl, 0, sizeof(Control), c->stream));
     return VPMC_OK;
 }
 
@@ -396,7 +391,6 @@ constexpr long long kMaxBatch = 1ll << 26;    // histories per devices -> patien
 
 vpmc_status grow_queries(vpmc_ctx* c, long long n)
 {
-    if (!c->d_sq_count) CUDA_TRY(dev_alloc(&c->d_sq_count, 1));
     if (n <= c->sq_cap) return VPMC_OK;
     cudaFree(c->d_sq);
     c->d_sq = nullptr;
@@ -425,19 +419,16 @@ vpmc_status enqueue_transport(vpmc_ctx* c, TransportParams p, long long total, c
     if (batch < 1) return fail(VPMC_ERR_STATE, "hand-off buffer smaller than one record per scenario");
     p.phase = c->d_phase;
     p.phase_cap = c->phase_cap;
-    p.phase_count = c->d_phase_count;
     p.rep_cap = batch;
     p.rep_hist = p.n_rep > 1 ? p.rep_hist : total;
     p.mid = c->d_mid;
     p.mid_cap = batch;
-    p.mid_count = c->d_mid_count;
     p.aggregate = t.aggregate;
     p.chunk = t.chunk;
     if (p.surrogate) {
         if (!c->d_sq || c->sq_cap < c->phase_cap) return fail(VPMC_ERR_STATE, "surrogate query buffer not sized");
         p.sq = c->d_sq;
         p.sq_cap = c->sq_cap;
-        p.sq_count = c->d_sq_count;
     }
     // the batch events are recorded as event nodes when the transport is
     // captured into a graph (external records), or directly otherwise
@@ -449,9 +440,7 @@ vpmc_status enqueue_transport(vpmc_ctx* c, TransportParams p, long long total, c
         const int b = c->kev_batches < vpmc_ctx::kTimedBatches ? c->kev_batches++ : -1;
         p.hist_begin = h0;
         p.total = std::min(total, h0 + batch);
-        CUDA_TRY(cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), c->stream));
-        CUDA_TRY(cudaMemsetAsync(c->d_phase_count, 0, sizeof(unsigned long long), c->stream));
-        if (p.surrogate) CUDA_TRY(cudaMemsetAsync(c->d_sq_count, 0, sizeof(unsigned long long), c->stream));
+        if (h0 > 0) CUDA_TRY(cudaMemsetAsync(c->d_ctl, 0, kControlBatchBytes, c->stream));   // (the first: reset_counters)
         if (b >= 0) CUDA_TRY(cudaEventRecordWithFlags(c->kev[3 * b], c->stream, rec_flags));
         CUDA_TRY(launch_devices(p, c->num_sms, t.dev_block, c->stream));
         if (p.surrogate) {
@@ -459,7 +448,6 @@ vpmc_status enqueue_transport(vpmc_ctx* c, TransportParams p, long long total, c
             CUDA_TRY(launch_sur_infer(c->sur, p, c->num_sms, c->stream));
             c->launches += 1;
         }
-        CUDA_TRY(cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), c->stream));
         if (b >= 0) CUDA_TRY(cudaEventRecordWithFlags(c->kev[3 * b + 1], c->stream, rec_flags));
         CUDA_TRY(launch_patient(p, c->num_sms, t.block, c->stream));
         if (b >= 0) CUDA_TRY(cudaEventRecordWithFlags(c->kev[3 * b + 2], c->stream, rec_flags));
@@ -482,10 +470,15 @@ vpmc_status add_kernel_times(vpmc_ctx* c, vpmc_stats* acc)
     return VPMC_OK;
 }
 
-vpmc_status read_stats(vpmc_ctx* c, int frac_bits, vpmc_stats* acc, bool add)
+// Waits for the stream's work and adds the call's counters (read in one copy,
+// with the status word) to acc.
+vpmc_status read_stats(vpmc_ctx* c, int frac_bits, vpmc_stats* acc, bool add, int* status)
 {
-    unsigned long long h[kNStats];
-    CUDA_TRY(cudaMemcpy(h, c->d_stats, sizeof h, cudaMemcpyDeviceToHost));
+    Control ctl;
+    CUDA_TRY(cudaMemcpyAsync(&ctl, c->d_ctl, sizeof ctl, cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
+    const unsigned long long* h = ctl.stats;
+    *status = ctl.status;
     const double sc = std::ldexp(1.0, -frac_bits);
     if (!add) *acc = vpmc_stats{};
     acc->e_dep += h[kStDep] * sc;
@@ -616,11 +609,7 @@ vpmc_status vpmc_create_geometry(vpmc_ctx** out, const int16_t* hu, int hu_on_de
     // from here on the CT holds the kernels' table index per voxel
     CTX_TRY(launch_ct_lut_index(c->d_ct, nct, c->stream));
     CTX_TRY(dev_alloc(&c->d_beams, kMaxBeams));
-    CTX_TRY(dev_alloc(&c->d_counter, 1));
-    CTX_TRY(dev_alloc(&c->d_phase_count, 1));
-    CTX_TRY(dev_alloc(&c->d_mid_count, 1));
-    CTX_TRY(dev_alloc(&c->d_stats, kNStats));
-    CTX_TRY(dev_alloc(&c->d_status, 1));
+    CTX_TRY(dev_alloc(&c->d_ctl, 1));
     CTX_TRY(dev_alloc(&c->d_scens, kMaxScen));
     CTX_TRY(cudaEventCreate(&c->ev0));
     CTX_TRY(cudaEventCreate(&c->ev1));
@@ -784,7 +773,6 @@ vpmc_status vpmc_run_spots(vpmc_ctx* c, const vpmc_spot* spots, int n_spots, con
         e_in += (double)s.n_hist * s.energy_mev;
     }
     if (qmax >= 9.0e18) return fail(VPMC_ERR_ARG, "fixed-point range exceeded: lower frac_bits or weights");
-    CUDA_TRY(cudaMemsetAsync(dose_dev, 0, c->nvox * sizeof(float), c->stream));
     if (!c->d_acc) CUDA_TRY(dev_alloc(&c->d_acc, c->nvox));
     CUDA_TRY(cudaMemsetAsync(c->d_acc, 0, c->nvox * sizeof(unsigned long long), c->stream));
     vpmc_stats stats{};
@@ -825,17 +813,16 @@ vpmc_status vpmc_run_spots(vpmc_ctx* c, const vpmc_spot* spots, int n_spots, con
     CUDA_TRY(launch_dose_normalise(c->d_acc, c->d_rho, c->nvox, scale, dose_dev, c->stream));
     ++c->launches;
     if (stats_out) {
-        CUDA_TRY(cudaStreamSynchronize(c->stream));
+        if (items.empty()) CUDA_TRY(cudaStreamSynchronize(c->stream));
         if (!items.empty()) {
-            st = read_stats(c, o.frac_bits, &stats, false);
+            int status = 0;
+            st = read_stats(c, o.frac_bits, &stats, false, &status);
             if (st != VPMC_OK) return st;
             float ms = 0.0f;
             CUDA_TRY(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
             stats.ms = ms;
             st = add_kernel_times(c, &stats);
             if (st != VPMC_OK) return st;
-            int status = 0;
-            CUDA_TRY(cudaMemcpy(&status, c->d_status, sizeof status, cudaMemcpyDeviceToHost));
             stats.histories = total;
             stats.e_in = e_in;
             stats.launches = c->launches - launches0;
@@ -1298,10 +1285,9 @@ vpmc_status vpmc_influence_matrix(vpmc_ctx* c, const vpmc_spot* spots, int n_spo
         float ms = 0.0f;
         IM_TRY(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
         total_ms += ms;
-        IM_ST(read_stats(c, o.frac_bits, &stats, true));
-        IM_ST(add_kernel_times(c, &stats));
         int status = 0;
-        IM_TRY(cudaMemcpy(&status, c->d_status, sizeof status, cudaMemcpyDeviceToHost));
+        IM_ST(read_stats(c, o.frac_bits, &stats, true, &status));
+        IM_ST(add_kernel_times(c, &stats));
         if (status & 1) {
             release();
             drop_outputs();
@@ -1491,21 +1477,16 @@ void vpmc_destroy(vpmc_ctx* c)
     cudaFree(c->d_raster_lb);
     cudaFree(c->d_raster_near);
     cudaFree(c->d_raster_local);
-    cudaFree(c->d_counter);
-    cudaFree(c->d_stats);
-    cudaFree(c->d_status);
+    cudaFree(c->d_ctl);
     cudaFree(c->d_scens);
     cudaFree(c->d_items);
     cudaFree(c->d_boxes);
     cudaFree(c->d_ovf);
     cudaFree(c->d_phase);
-    cudaFree(c->d_phase_count);
     cudaFree(c->d_mid);
-    cudaFree(c->d_mid_count);
     cudaFree(c->d_scratch);
     cudaFree(c->d_poly_kappa);
     cudaFree(c->d_sq);
-    cudaFree(c->d_sq_count);
     cudaFree(c->sur.params);
     cudaFree(c->sur.grad);
     cudaFree(c->sur.gpart);
@@ -1779,13 +1760,10 @@ vpmc_status vpmc_surrogate_tracks(vpmc_ctx* c, const int* beam_ids, int n_beams,
     p.surrogate = use_surrogate ? 1 : 0;
     p.sq = c->d_sq;
     p.sq_cap = c->sq_cap;
-    p.sq_count = c->d_sq_count;
     p.phase = c->d_phase;
     p.phase_cap = c->phase_cap;
-    p.phase_count = c->d_phase_count;
     p.mid = c->d_mid;
     p.mid_cap = c->phase_cap;
-    p.mid_count = c->d_mid_count;
     p.aggregate = 0;
     p.chunk = 32;
     st = reset_counters(c);
@@ -1796,8 +1774,7 @@ vpmc_status vpmc_surrogate_tracks(vpmc_ctx* c, const int* beam_ids, int n_beams,
     for (long long h0 = 0; h0 < total; h0 += batch) {
         p.hist_begin = h0;
         p.total = std::min(total, h0 + batch);
-        cudaError_t e = cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), c->stream);
-        if (e == cudaSuccess && use_surrogate) e = cudaMemsetAsync(c->d_sq_count, 0, sizeof(unsigned long long), c->stream);
+        cudaError_t e = h0 > 0 ? cudaMemsetAsync(c->d_ctl, 0, kControlBatchBytes, c->stream) : cudaSuccess;
         if (e == cudaSuccess) e = launch_devices(p, c->num_sms, block, c->stream);
         if (e == cudaSuccess && use_surrogate) e = launch_sur_infer(c->sur, p, c->num_sms, c->stream);
         if (e != cudaSuccess) return done(fail(VPMC_ERR_CUDA, "track launch: %s", cudaGetErrorString(e)));
@@ -1806,7 +1783,7 @@ vpmc_status vpmc_surrogate_tracks(vpmc_ctx* c, const int* beam_ids, int n_beams,
     if (cudaStreamSynchronize(c->stream) != cudaSuccess)
         return done(fail(VPMC_ERR_CUDA, "track transport: %s", cudaGetErrorString(cudaGetLastError())));
     int status = 0;
-    if (cudaMemcpy(&status, c->d_status, sizeof status, cudaMemcpyDeviceToHost) != cudaSuccess)
+    if (cudaMemcpy(&status, &c->d_ctl->status, sizeof status, cudaMemcpyDeviceToHost) != cudaSuccess)
         return done(fail(VPMC_ERR_CUDA, "status read failed"));
     if (status & 1) return done(fail(VPMC_ERR_TIMEOUT, "tracks reached the iteration cap"));
     if (status & 6) return done(fail(VPMC_ERR_DEVICE_FLAG, "query buffer overflow (status %d)", status));

@@ -76,9 +76,7 @@ struct vpmc_ctx {
     uint16_t* d_raster_near = nullptr;
     uint32_t* d_raster_local = nullptr;
     // per-launch buffers
-    unsigned long long* d_counter = nullptr;
-    unsigned long long* d_stats = nullptr;
-    int* d_status = nullptr;
+    vpmc::Control* d_ctl = nullptr;
     vpmc::DevScen* d_scens = nullptr;
     vpmc::DevItem* d_items = nullptr;
     size_t items_cap = 0;
@@ -89,8 +87,6 @@ struct vpmc_ctx {
     vpmc::PhaseRec* d_phase = nullptr;               // hand-off from the aperture to the patient kernel
     vpmc::PhaseRec* d_mid = nullptr;                 // hand-off from the range-shifter to the aperture kernel
     long long phase_cap = 0;                         // records of each hand-off buffer
-    unsigned long long* d_phase_count = nullptr;
-    unsigned long long* d_mid_count = nullptr;
     unsigned long long* d_scratch = nullptr;
     size_t scratch_cap = 0;                    // elements
     float* d_poly_kappa = nullptr;             // per polygon vertex: signed curvature (surrogate inputs)
@@ -100,7 +96,6 @@ struct vpmc_ctx {
     int sur_step = 0;                          // Adam steps taken since the weights were set
     vpmc::SurQuery* d_sq = nullptr;            // brass entries handed to the surrogate
     long long sq_cap = 0;
-    unsigned long long* d_sq_count = nullptr;
     long long launches = 0;                    // kernels launched since creation
     // per transport batch: events before the beam-line kernels, between them
     // and the patient kernel, and after it (the first kTimedBatches batches)

@@ -291,9 +291,9 @@ __global__ void __launch_bounds__(768, 1) k_source_rs(const TransportParams P)
         float2* R = reinterpret_cast<float2*>(smem + SourceSmem::R);
         float2* Et = reinterpret_cast<float2*>(smem + SourceSmem::Einv);
 #pragma unroll 1
-        for (int i = threadIdx.x; i < kNEPad; i += blockDim.x) R[i] = P.tables->R[kPMMA][i];
+        for (int i = P.any_rs ? threadIdx.x : kNEPad; i < kNEPad; i += blockDim.x) R[i] = P.tables->R[kPMMA][i];
 #pragma unroll 1
-        for (int i = threadIdx.x; i < kNR; i += blockDim.x) Et[i] = P.tables->Einv[kPMMA][i];
+        for (int i = P.any_rs ? threadIdx.x : kNR; i < kNR; i += blockDim.x) Et[i] = P.tables->Einv[kPMMA][i];
         MatConst* mt = reinterpret_cast<MatConst*>(smem + SourceSmem::Mat);
         if (threadIdx.x < kNMat) mt[threadIdx.x] = P.tables->mat[threadIdx.x];
         DevBeam* bm = reinterpret_cast<DevBeam*>(smem + SourceSmem::Beams);
@@ -493,9 +493,9 @@ __global__ void __launch_bounds__(768, 1) k_aperture(const TransportParams P)
         float2* R = reinterpret_cast<float2*>(smem + ApertureSmem::R);
         float2* Et = reinterpret_cast<float2*>(smem + ApertureSmem::Einv);
 #pragma unroll 1
-        for (int i = threadIdx.x; i < kNEPad; i += blockDim.x) R[i] = P.tables->R[kBrass][i];
+        for (int i = P.any_ap ? threadIdx.x : kNEPad; i < kNEPad; i += blockDim.x) R[i] = P.tables->R[kBrass][i];
 #pragma unroll 1
-        for (int i = threadIdx.x; i < kNR; i += blockDim.x) Et[i] = P.tables->Einv[kBrass][i];
+        for (int i = P.any_ap ? threadIdx.x : kNR; i < kNR; i += blockDim.x) Et[i] = P.tables->Einv[kBrass][i];
         MatConst* mt = reinterpret_cast<MatConst*>(smem + ApertureSmem::Mat);
         if (threadIdx.x < kNMat) mt[threadIdx.x] = P.tables->mat[threadIdx.x];
         DevBeam* bm = reinterpret_cast<DevBeam*>(smem + ApertureSmem::Beams);
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(768, 1) k_aperture(const TransportParams P)
         for (int i = threadIdx.x; i < P.n_scen; i += blockDim.x) sc[i] = P.scens[i];
         float2* pl = reinterpret_cast<float2*>(smem + ApertureSmem::Poly);
 #pragma unroll 1
-        for (int i = threadIdx.x; i < P.n_poly; i += blockDim.x) pl[i] = P.poly[i];
+        for (int i = P.any_ap ? threadIdx.x : P.n_poly; i < P.n_poly; i += blockDim.x) pl[i] = P.poly[i];
     }
     __syncthreads();
     const MatConst* mat = reinterpret_cast<const MatConst*>(smem + ApertureSmem::Mat);
@@ -962,20 +962,20 @@ static cudaError_t launch_source_rs(const TransportParams& p, int grid, cudaStre
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    k_source_rs<kAllPhysics><<<grid, 768, SourceSmem::Bytes, s>>>(p);      // 78 registers: 768 threads fit
+    k_source_rs<kAllPhysics><<<grid, spread_block(p, p.total - p.hist_begin, grid, 768), SourceSmem::Bytes, s>>>(p);   // 78 registers: 768 threads fit
     return cudaGetLastError();
 }
 
-cudaError_t launch_devices(const TransportParams& p, int grid, int block, cudaStream_t s)
+cudaError_t launch_devices(TransportParams p, int grid, int block, cudaStream_t s)
 {
     const int mode = (p.surrogate ? 1 : 0) | (p.track_mode ? 2 : 0);
+    p.counter = &p.work[0].taken;
+    block = spread_block(p, p.total - p.hist_begin, grid, block);
     if (!p.track_mode) {
-        cudaError_t e = cudaMemsetAsync(p.mid_count, 0, sizeof(unsigned long long), s);
+        const cudaError_t e = (p.mcs && p.straggling && p.nuclear && p.fx32) ? launch_source_rs<true>(p, grid, s) : launch_source_rs<false>(p, grid, s);
         if (e != cudaSuccess) return e;
-        e = (p.mcs && p.straggling && p.nuclear && p.fx32) ? launch_source_rs<true>(p, grid, s) : launch_source_rs<false>(p, grid, s);
-        if (e != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(p.counter, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
     }
+    p.counter = &p.work[1].taken;
     switch (mode) {
     case 1: return launch_aperture_mode<1>(p, grid, block, s);
     case 2: return launch_aperture_mode<2>(p, grid, block, s);

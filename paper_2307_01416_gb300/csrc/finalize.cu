@@ -55,7 +55,7 @@ __global__ void k_dose_normalise(const unsigned long long* __restrict__ acc, con
 {
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nvox;
          v += (long long)gridDim.x * blockDim.x)
-        dose[v] = (float)((double)acc[v] * scale / rho[v]);
+        dose[v] = acc[v] ? (float)((double)acc[v] * scale / rho[v]) : 0.0f;   // most voxels: no FP64 division
 }
 
 // FP32 screen of the FP64 quotient q / rho: q's two 32-bit halves converted

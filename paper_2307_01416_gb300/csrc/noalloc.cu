@@ -33,9 +33,8 @@ constexpr size_t kOffBox = kOffItems + align256(sizeof(DevItem) * kMaxItems);
 constexpr size_t kOffScen = kOffBox + align256(sizeof(DevBox));
 constexpr size_t kOffPhase = kOffScen + align256(sizeof(DevScen));
 constexpr size_t kOffMid = kOffPhase + align256(sizeof(PhaseRec) * kBatch);
-constexpr size_t kOffCount = kOffMid + align256(sizeof(PhaseRec) * kBatch);      // counter, two hand-off counts, stats
-constexpr size_t kOffStatus = kOffCount + align256(sizeof(unsigned long long) * (3 + kNStats));
-constexpr size_t kScratchBytes = kOffStatus + 256;                              // about 29 MiB
+constexpr size_t kOffCtl = kOffMid + align256(sizeof(PhaseRec) * kBatch);
+constexpr size_t kScratchBytes = kOffCtl + align256(sizeof(Control));           // about 29 MiB
 
 // The scratch of every call on a device (each GPU that loads the library
 // holds it until the process exits).
@@ -94,7 +93,7 @@ vpmc_status pending_status(int device, cudaStream_t stream)
     int st_word = 0;
     if (s == stream) NA_TRY(cudaStreamSynchronize(stream));
     else NA_TRY(cudaDeviceSynchronize());
-    NA_TRY(cudaMemcpyAsync(&st_word, g_addr[device] + kOffStatus, sizeof st_word, cudaMemcpyDeviceToHost, stream));
+    NA_TRY(cudaMemcpyAsync(&st_word, g_addr[device] + kOffCtl + offsetof(Control, status), sizeof st_word, cudaMemcpyDeviceToHost, stream));
     NA_TRY(cudaStreamSynchronize(stream));
     if (st_word & 1)
         return report_error(VPMC_ERR_TIMEOUT, "an earlier asynchronous call: histories reached the iteration cap");
@@ -156,8 +155,7 @@ extern "C" vpmc_status vpmc_run_spots_noalloc(vpmc_ctx* c, const vpmc_spot* spot
     DevScen* dscen = reinterpret_cast<DevScen*>(base + kOffScen);
     PhaseRec* phase = reinterpret_cast<PhaseRec*>(base + kOffPhase);
     PhaseRec* mid = reinterpret_cast<PhaseRec*>(base + kOffMid);
-    unsigned long long* counters = reinterpret_cast<unsigned long long*>(base + kOffCount);
-    int* status = reinterpret_cast<int*>(base + kOffStatus);
+    Control* ctl = reinterpret_cast<Control*>(base + kOffCtl);
 
     // work items, uploaded from a small stack buffer (pageable copies are
     // staged before cudaMemcpyAsync returns, so the buffer can be reused)
@@ -216,9 +214,7 @@ extern "C" vpmc_status vpmc_run_spots_noalloc(vpmc_ctx* c, const vpmc_spot* spot
     NA_TRY(cudaMemcpyAsync(dscen, &sc, sizeof sc, cudaMemcpyHostToDevice, c->stream));
     // the array keeps the previous call's contents: clear what must start at zero
     NA_TRY(cudaMemsetAsync(acc, 0, (size_t)c->nvox * sizeof(unsigned long long), c->stream));
-    NA_TRY(cudaMemsetAsync(counters, 0, sizeof(unsigned long long) * (3 + kNStats), c->stream));
-    NA_TRY(cudaMemsetAsync(status, 0, sizeof(int), c->stream));
-    NA_TRY(cudaMemsetAsync(dose_dev, 0, (size_t)c->nvox * sizeof(float), c->stream));
+    NA_TRY(cudaMemsetAsync(ctl, 0, sizeof(Control), c->stream));
 
     TransportParams p{};
     p.tables = c->d_tables;
@@ -241,11 +237,8 @@ extern "C" vpmc_status vpmc_run_spots_noalloc(vpmc_ctx* c, const vpmc_spot* spot
     p.items = items;
     p.n_items = n_items;
     p.boxes = box;
-    p.counter = counters;
-    p.phase_count = counters + 1;
-    p.mid_count = counters + 2;
-    p.stats = counters + 3;
-    p.status = status;
+    set_control(&p, ctl);
+    beam_flags(&p, c->beams, kMaxBeams);
     p.scratch = acc;
     p.unit_weight = unit_weight ? 1 : 0;
     p.phase = phase;
@@ -272,10 +265,8 @@ extern "C" vpmc_status vpmc_run_spots_noalloc(vpmc_ctx* c, const vpmc_spot* spot
     for (long long h0 = 0; h0 < total; h0 += kBatch) {
         p.hist_begin = h0;
         p.total = h0 + kBatch < total ? h0 + kBatch : total;
-        NA_TRY(cudaMemsetAsync(p.counter, 0, sizeof(unsigned long long), c->stream));
-        NA_TRY(cudaMemsetAsync(p.phase_count, 0, sizeof(unsigned long long), c->stream));
+        if (h0 > 0) NA_TRY(cudaMemsetAsync(ctl, 0, kControlBatchBytes, c->stream));   // (the first: above)
         NA_TRY(launch_devices(p, c->num_sms, t.dev_block, c->stream));
-        NA_TRY(cudaMemsetAsync(p.counter, 0, sizeof(unsigned long long), c->stream));
         NA_TRY(launch_patient(p, c->num_sms, t.block, c->stream));
         c->launches += 3;
     }
@@ -290,12 +281,11 @@ extern "C" vpmc_status vpmc_run_spots_noalloc(vpmc_ctx* c, const vpmc_spot* spot
         g_pending[device].stream = c->stream;
     }
     if (stats_out) {
+        Control h;
+        NA_TRY(cudaMemcpyAsync(&h, ctl, sizeof h, cudaMemcpyDeviceToHost, c->stream));
         NA_TRY(cudaStreamSynchronize(c->stream));
-        unsigned long long h[3 + kNStats];
-        int st_word = 0;
-        NA_TRY(cudaMemcpy(h, counters, sizeof h, cudaMemcpyDeviceToHost));
-        NA_TRY(cudaMemcpy(&st_word, status, sizeof st_word, cudaMemcpyDeviceToHost));
-        const unsigned long long* v = h + 3;
+        const int st_word = h.status;
+        const unsigned long long* v = h.stats;
         const double q = std::ldexp(1.0, -o.frac_bits);
         vpmc_stats r;
         std::memset(&r, 0, sizeof r);

@@ -384,8 +384,10 @@ int patient_nest_variant(const int nest_shift[3])
     return mask == 7 ? 7 : ((mask & 3) == 3 ? 3 : 0);
 }
 
-cudaError_t launch_patient(const TransportParams& p, int grid, int block, cudaStream_t s)
+cudaError_t launch_patient(TransportParams p, int grid, int block, cudaStream_t s)
 {
+    p.counter = &p.work[2].taken;
+    block = spread_block(p, (p.total - p.hist_begin) * p.n_rep, grid, block);
     switch (patient_nest_variant(p.nest_shift)) {
     case 7: return launch_patient_nest<7>(p, grid, block, s);
     case 3: return launch_patient_nest<3>(p, grid, block, s);

@@ -161,6 +161,22 @@ struct HistRecord {                  // mirrors vpmc_history_record
     float pad;
 };
 
+// Counters of a transport call, one allocation: reset by one memset before the
+// call, its first part before every further batch, and read by one copy.  Each
+// work counter has a 128-byte line of its own: an atomic evicts its line from
+// the SM's L1, and the hand-off counts are read at every refill (all counters
+// in one line: 0.2 ms more on 2e5 histories in water, 7 ms on 1.6e8).
+struct WorkCounter {
+    unsigned long long taken, pad[15];
+};
+struct Control {
+    WorkCounter work[3];             // work taken by k_source_rs, k_aperture, k_patient
+    unsigned long long mid_count, phase_count, sq_count, pad[13];
+    unsigned long long stats[kNStats];
+    int status;
+};
+constexpr size_t kControlBatchBytes = offsetof(Control, stats);
+
 struct TransportParams {
     const TablesImage* tables;
     const uint16_t* ct_lut;          // per CT voxel: index into the (density, SPR) table
@@ -182,7 +198,9 @@ struct TransportParams {
     int n_items;
     const DevBox* boxes;
     long long total;                 // total histories
-    unsigned long long* counter;     // global work counter
+    unsigned long long* counter;     // work taken by this kernel (set from `work` by the launch)
+    WorkCounter* work;               // [3]: source, aperture, patient
+    int any_rs, any_ap;              // some item's field has a range shifter, an aperture
     unsigned long long* scratch;     // deposit target
     long long hist_begin;            // beam-line kernels: first global history of the batch
     PhaseRec* mid;                   // histories handed from the range-shifter to the aperture kernel (BEV)
@@ -290,13 +308,48 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned block, size_t
 }
 
 // Host-side launchers (transport.cu, finalize.cu).
+// Threads per block of a persistent launch over at most n histories: warps that
+// the work cannot fill are left out, so that every SM gets some of it.  With
+// full blocks the first ones to have staged their tables take all of a small
+// launch, 28 warps each, and their SMs' issue slots set its time: 2,000
+// histories in water 350 us in the patient kernel at 896 threads (400 at 512,
+// 290 at 256), 250 us at 128; 2,000 behind range shifter and aperture 0.58 ms in
+// the beam-line kernels, 0.59 at full blocks.  Not below 128: the block stages
+// its tables.
+inline int spread_block(const TransportParams& p, long long n, int grid, int block)
+{
+    const long long chunks = (n + p.chunk - 1) / p.chunk;
+    const long long warps = (chunks + grid - 1) / grid;
+    const long long fit = warps > 4 ? 32 * warps : 128;
+    return fit < block ? (int)fit : block;
+}
+
+inline void set_control(TransportParams* p, Control* ctl)
+{
+    p->work = ctl->work;
+    p->mid_count = &ctl->mid_count;
+    p->phase_count = &ctl->phase_count;
+    p->sq_count = &ctl->sq_count;
+    p->stats = ctl->stats;
+    p->status = &ctl->status;
+}
+
+// Which of the beam-line tables the beams need: the kernels stage only these.
+inline void beam_flags(TransportParams* p, const DevBeam* beams, int n)
+{
+    p->any_rs = p->any_ap = 0;
+    for (int b = 0; b < n; ++b) {
+        p->any_rs |= beams[b].rs;
+        p->any_ap |= beams[b].ap;
+    }
+}
+
 // Transport of histories [p.hist_begin, p.total): the beam-line kernels
-// (source and range shifter, then the aperture: launch_devices, which resets
-// p.counter between them), then the patient kernel on the histories they hand
-// over (p.mid and p.phase must each hold p.total - p.hist_begin records).
+// (source and range shifter, then the aperture: launch_devices), then the
+// patient kernel on the histories they hand over (p.mid and p.phase must each hold p.total - p.hist_begin records).
 // All launches are persistent grids of one block per SM.
-cudaError_t launch_devices(const TransportParams& p, int grid, int block, cudaStream_t s);
-cudaError_t launch_patient(const TransportParams& p, int grid, int block, cudaStream_t s);
+cudaError_t launch_devices(TransportParams p, int grid, int block, cudaStream_t s);
+cudaError_t launch_patient(TransportParams p, int grid, int block, cudaStream_t s);
 // Which compiled nesting of the patient kernel serves these grids (bit k: axis k nested).
 int patient_nest_variant(const int nest_shift[3]);
 // Converts a device CT of hounsfield units, in place, to indices into the
