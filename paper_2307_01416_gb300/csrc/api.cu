@@ -1024,6 +1024,7 @@ vpmc_status vpmc_influence_matrix(vpmc_ctx* c, const vpmc_spot* spots, int n_spo
     std::vector<float> reach((size_t)n_scen * nr, 0.0f);
     {
         std::vector<DepthJob> jobs;
+        int max_columns = 1;
         std::vector<float> rl;
         std::vector<int> slot((size_t)n_scen * nr);     // (scenario, run) -> entry of rl / reach
         for (int s = 0; s < n_scen; ++s)
@@ -1047,6 +1048,7 @@ vpmc_status vpmc_influence_matrix(vpmc_ctx* c, const vpmc_spot* spots, int n_spo
                 J.da = (float)da;
                 J.na = std::max(1, (int)std::ceil((f.a1 - f.a0 + 2 * lat) / da) + 1);
                 J.nb = std::max(1, (int)std::ceil((f.b1 - f.b0 + 2 * lat) / da) + 1);
+                max_columns = std::max(max_columns, J.na * J.nb);
                 J.t0 = (float)f.t0;
                 J.t1 = (float)f.t1;
                 J.dt = 0.5f;
@@ -1073,7 +1075,7 @@ vpmc_status vpmc_influence_matrix(vpmc_ctx* c, const vpmc_spot* spots, int n_spo
         if (e == cudaSuccess) e = cudaMemsetAsync(d_reach, 0, rl.size() * sizeof(unsigned), c->stream);
         if (e == cudaSuccess)
             e = launch_depth_bounds(reinterpret_cast<const uint16_t*>(c->d_ct), c->d_tables, c->ctg, d_jobs,
-                                    (int)jobs.size(), d_rl, d_reach, c->stream);
+                                    (int)jobs.size(), max_columns, d_rl, d_reach, c->stream);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(h_reach.data(), d_reach, rl.size() * sizeof(unsigned), cudaMemcpyDeviceToHost,
                                 c->stream);

@@ -478,9 +478,10 @@ struct DepthJob {
     int run_off, run_n;
 };
 // reach[run] (FP32 bits, zeroed by the caller): the largest t - t0 over the
-// columns at which the water-equivalent path reaches r_lim[run].
+// columns at which the water-equivalent path reaches r_lim[run].  max_columns:
+// the largest na x nb of the jobs (the launch's size; any value is correct).
 cudaError_t launch_depth_bounds(const uint16_t* ct, const TablesImage* tables, Grid3 ctg, const DepthJob* jobs,
-                                int n_jobs, const float* r_lim, unsigned* reach, cudaStream_t s);
+                                int n_jobs, int max_columns, const float* r_lim, unsigned* reach, cudaStream_t s);
 // Counting sort of out-of-box records into per-(scenario, voxel) buckets,
 // then per bucket: sort by item, merge duplicates, raise the column maxima.
 cudaError_t launch_ovf_count(const OvfRec* rec, long long n, int n_spots, long long nvox, long long* bucket_cnt,
