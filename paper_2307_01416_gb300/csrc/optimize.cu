@@ -35,7 +35,7 @@ namespace {
 
 constexpr unsigned kFullMask = 0xffffffffu;
 constexpr int kLanesPerRow = 8;                 // full-matrix products: 4 rows per warp
-constexpr int kSpmvBlocks = 8;                  // full-matrix products: blocks per SM and matrix
+constexpr int kSpmvBlocks = 16;                 // full-matrix products: blocks per SM and matrix
 
 struct Csr {
     const long long* row_ptr;
@@ -91,7 +91,11 @@ struct IndexSums {
 // in flight per lane, and the next row's pointers are read before this row's
 // entries are used, since most rows are shorter than one batch of the
 // sub-warp and the chain pointers -> entries -> weights would be their time.
-// 13 matrices of 6.4e7 entries: 3.1 ms with one entry per lane in flight.
+// 13 matrices of 6.4e7 entries: 3.1 ms with one entry per lane in flight,
+// 1.63 ms with eight and an even number of warps, 1.36 ms with an odd one (one
+// matrix 172 -> 140 us).  Batches of 4, 6, 12, 16: 1.88, 1.74, 1.48, 1.71 ms;
+// the weights staged in shared memory (two blocks of 512 threads per SM) 1.69;
+// a warp on each row of more than 32 entries 2.6.
 constexpr int kBatch = 8;
 template <bool kIndices>
 __global__ void __launch_bounds__(256) k_spmv(const __grid_constant__ CsrSet mats, long long n_rows, int n_cols,
@@ -101,7 +105,9 @@ __global__ void __launch_bounds__(256) k_spmv(const __grid_constant__ CsrSet mat
     const Csr A = mats.m[blockIdx.y];
     const int lane = threadIdx.x & 31, sub = lane & (kLanesPerRow - 1);
     constexpr int kRowsPerWarp = 32 / kLanesPerRow;
-    const long long wstride = (long long)gridDim.x * (blockDim.x >> 5) * kRowsPerWarp;
+    // an odd number of warps: rows of one phase of a grid whose width is a power
+    // of two times 4 are all inside the field or all empty
+    const long long wstride = (((long long)gridDim.x * (blockDim.x >> 5) - 1) | 1) * kRowsPerWarp;
     unsigned hit = 0, target = 0, high = 0;
     int mn = kMaxBits, mx = 0;
     // warp-uniform loop over groups of kRowsPerWarp rows (the shuffles below
@@ -115,6 +121,7 @@ __global__ void __launch_bounds__(256) k_spmv(const __grid_constant__ CsrSet mat
             e = __ldg(A.row_ptr + row + 1);
         }
     };
+    if (base >= wstride) base = n_rows;                // (the warp too many)
     row_bounds(base + lane / kLanesPerRow);
     for (; base < n_rows; base += wstride) {
         const long long row = base + lane / kLanesPerRow;
