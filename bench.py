@@ -402,8 +402,8 @@ def main():
                               "achieved": adds_rate, "peak": l2["adds_per_s"],
                               "frac": adds_rate / l2["adds_per_s"] if adds_rate else None,
                               "k_patient_ms_per_step": ms_patient / args.steps,
-                              "note": "one 64-bit scoring add per patient step (plain atomics; warp aggregation "
-                                      "would issue fewer) over k_patient's CUDA-event time; peak = "
+                              "note": "upper bound: one 64-bit scoring add per patient step (the kernel adds once "
+                                      "per voxel visit) over k_patient's CUDA-event time; peak = "
                                       "vpmc_measure_l2_atomics over a 32 MiB buffer"}}
         e2e = _leg(lambda: e2e_leg(pb, spots, scens, opts, args), not args.no_e2e)
         cpu = _leg(lambda: cpu_baseline(pb, spots, args.cpu_seconds), not args.no_cpu_baseline and world == 1)
