@@ -15,10 +15,11 @@ namespace vpmc {
 // one shape for every call, a full block per SM and chunks of one warp.  With
 // a deposit per voxel visit (patient.cu) it is the fastest of blocks of 512
 // to 896 threads, plain or warp-aggregated atomics and chunks of 16 to 128 on
-// every workload measured, or within 1 % of it (3.2e7 histories in the head:
-// 134 ms at 896 threads, 135 at 768, 162 at 512; aggregated atomics 227 ms;
-// chunks of 128 134.6 ms there and 4.6 against 4.1 ms on 4e6 histories behind
-// an aperture), so nothing is timed before a context's first call.
+// every workload measured, or within 1 % of it (k_patient on 3.2e7 histories in
+// the head: 121.6 ms at 896 threads, 123.5 at 768, 136.9 at 512; aggregated
+// atomics 219.9 ms; chunks of 128 122.2 ms there and 4.3 against 3.8 ms on 4e6
+// histories behind an aperture; chunks of 16 a third slower in the beam-line
+// kernels), so nothing is timed before a context's first call.
 struct LaunchShape {
     int dev_block = 768;     // k_aperture threads per block (a full block)
     int block = 896;         // k_patient threads per block
