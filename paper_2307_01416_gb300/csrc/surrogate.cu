@@ -58,6 +58,12 @@ constexpr bool w3p_is_inverse()
 static_assert(w3p_is_inverse(), "the training order holds every output");
 constexpr int kWaitLimit = 1 << 22;       // mbarrier polls before a wait is declared failed
 
+// What a wait returns.  A test replaces it to let one thread's wait fail
+// although the work it waited for is complete.
+#ifndef VPMC_WAIT_RESULT
+#define VPMC_WAIT_RESULT(mbar, parity, done) (done)
+#endif
+
 // Byte offset of element (r, k) of an R x K operand in the no-swizzle
 // K-major layout: core matrix (r / 8, k / 8) of 8 rows x 16 bytes.
 __host__ __device__ constexpr int kmaj(int r, int k, int K)
@@ -111,15 +117,13 @@ __device__ __forceinline__ void mbar_init(uint32_t mbar)
 // Bounded wait for the completion of the mbarrier phase with the given parity.
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity)
 {
-    for (int i = 0; i < kWaitLimit; ++i) {
-        uint32_t done;
+    uint32_t done = 0u;
+    for (int i = 0; i < kWaitLimit && !done; ++i)
         asm volatile(
             "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}\n"
             : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
-        if (done) return true;
-    }
-    return false;
+    return VPMC_WAIT_RESULT(mbar, parity, done != 0u);
 }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t slot_saddr, uint32_t ncols)
@@ -255,13 +259,27 @@ __device__ __forceinline__ void mma_operands(uint32_t d_tmem, Operand A, Operand
     }
 }
 
+// Waits, as one warp, for the work committed to mbar last.  The parity moves on
+// only when that work is complete: after a failed wait it still names the phase
+// that is open, so that the kernel's end can wait for it once more.
+__device__ __forceinline__ bool work_done(uint32_t mbar, uint32_t& parity)
+{
+    const bool done = __all_sync(kFull, mbar_wait(mbar, parity));
+    if (done) parity ^= 1u;
+    tc_fence_after();
+    return done;
+}
+
 // Make this thread's generic-proxy shared-memory writes and tensor-memory
-// reads visible to the next tensor-core operation, then synchronise.
-__device__ __forceinline__ void publish()
+// reads visible to the next tensor-core operation, then synchronise.  Returns
+// whether every thread passed ok: work is issued only when none of the waits
+// before it failed, so at most one phase is ever open and nobody touches the
+// operands of work in flight.
+__device__ __forceinline__ bool publish(bool ok)
 {
     fence_async_smem();
     tc_fence_before();
-    __syncthreads();
+    return __syncthreads_and(ok) != 0;
 }
 
 // Barrier of one 128-thread warpgroup (named barrier 1 + g): the forward
@@ -284,11 +302,11 @@ __device__ __forceinline__ bool group_sync_and(int g, bool ok)
 }
 
 // publish for one warpgroup's tile pipeline.
-__device__ __forceinline__ void publish_group(int g)
+__device__ __forceinline__ bool publish_group(int g, bool ok)
 {
     fence_async_smem();
     tc_fence_before();
-    group_sync(g);
+    return group_sync_and(g, ok);
 }
 
 __device__ __forceinline__ void copy_to_smem(unsigned char* dst, const unsigned char* src, int bytes)
@@ -431,11 +449,11 @@ using FwdS = FwdSmem<kFwdGroups, false>;
 using InferS = FwdSmem<kInferGroups, true>;
 constexpr uint32_t kFwdCols = 512;        // allocation (a power of two); group g uses columns [128 g, 128 g + 128)
 
-// The three GEMMs of one tile whose inputs are in the group's X and published;
-// clears ok when a tensor-core wait failed (the caller's group agrees on it).
-// On return the group's accumulator columns hold z - b3.
+// The three GEMMs of one tile whose inputs are in the group's X and published.
+// On return the group's accumulator columns hold z - b3, unless ok is false in
+// this warp (its wait failed) or the call returned false (the group stopped).
 template <class S>
-__device__ __forceinline__ void forward_tile(unsigned char* sm, unsigned char* gs, uint32_t tcol, uint32_t t_row,
+__device__ __forceinline__ bool forward_tile(unsigned char* sm, unsigned char* gs, uint32_t tcol, uint32_t t_row,
                                              uint32_t& phase, int r, int g, bool& ok)
 {
     const uint32_t s0 = smem_addr(sm), gs0 = smem_addr(gs), bar = gs0 + S::Bar;
@@ -445,29 +463,24 @@ __device__ __forceinline__ void forward_tile(unsigned char* sm, unsigned char* g
         mma_tile(tcol, gs0 + S::X, s0 + S::W + kImgW1, kInPad, kH, false);
         umma_commit(bar);
     }
-    ok = mbar_wait(bar, phase) && ok;
-    phase ^= 1u;
-    tc_fence_after();
-    hidden_epilogue_fwd(t_row, bias, gs + S::H, r);
-    publish_group(g);
+    ok = work_done(bar, phase);
+    if (ok) hidden_epilogue_fwd(t_row, bias, gs + S::H, r);
+    if (!publish_group(g, ok)) return false;
     if (r == 0) {
         tc_fence_after();
         mma_tile(tcol, gs0 + S::H, s0 + S::W + kImgW2, kH, kH, false);
         umma_commit(bar);
     }
-    ok = mbar_wait(bar, phase) && ok;
-    phase ^= 1u;
-    tc_fence_after();
-    hidden_epilogue_fwd(t_row, bias + kH, gs + S::H, r);
-    publish_group(g);
+    ok = work_done(bar, phase);
+    if (ok) hidden_epilogue_fwd(t_row, bias + kH, gs + S::H, r);
+    if (!publish_group(g, ok)) return false;
     if (r == 0) {
         tc_fence_after();
         mma_tile(tcol, gs0 + S::H, s0 + S::W + kImgW3, kH, kOutPad, false);
         umma_commit(bar);
     }
-    ok = mbar_wait(bar, phase) && ok;
-    phase ^= 1u;
-    tc_fence_after();
+    ok = work_done(bar, phase);
+    return true;
 }
 
 template <class S, int kG>
@@ -493,10 +506,10 @@ __device__ __forceinline__ void fwd_epilogue_free(unsigned char* sm, uint32_t tb
                                                   bool ok, const SurNet& net)
 {
     if (!ok) {
-        // a wait failed: latch the error and give the tensor core a last
-        // bounded chance to finish this group's work before the memory is
-        // released
-        if ((threadIdx.x & (kRows - 1)) == 0) atomicOr(net.status, 1);
+        // a wait failed in this warp: latch the error and give the tensor core
+        // a last bounded chance to finish this group's work before the memory
+        // is released
+        atomicOr(net.status, 1);
         (void)mbar_wait(bar, phase);
     }
     tc_fence_before();
@@ -549,24 +562,23 @@ __global__ void __launch_bounds__(kFwdGroups * kRows, 1) k_sur_forward(const Sur
         }
         store_input_row(gs + S::X, r, f);
         if (r == 0) bulk_store_wait_read();         // the last outputs have left the staging tile
-        fence_async_smem();
-        tc_fence_before();
-        ok = group_sync_and(g, ok);                 // publishes X; the group agrees on the waits so far
-        if (!ok) break;
+        if (!publish_group(g, ok)) break;
         loading = whole(tile + stride);
         if (loading && r == 0)
             bulk_load(smem_addr(xs), x + kIn * kRows * (tile + stride), kRows * kIn * 4, bar_in);
-        forward_tile<S>(sm, gs, tcol, t_row, phase, r, g, ok);
+        if (!forward_tile<S>(sm, gs, tcol, t_row, phase, r, g, ok)) break;
         // outputs through shared memory (h2 is consumed): rows x 45 contiguous
         // floats (row0 * 180 bytes is a multiple of 16)
-        float v[32], u[16];
-        tmem_ld32(t_row, v);
-        tmem_ld16(t_row + 32u, u);
+        if (ok) {
+            float v[32], u[16];
+            tmem_ld32(t_row, v);
+            tmem_ld16(t_row + 32u, u);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) zs[kOut * r + j] = v[j] + b3[j];
+            for (int j = 0; j < 32; ++j) zs[kOut * r + j] = v[j] + b3[j];
 #pragma unroll
-        for (int j = 32; j < kOut; ++j) zs[kOut * r + j] = u[j - 32] + b3[j];
-        publish_group(g);
+            for (int j = 32; j < kOut; ++j) zs[kOut * r + j] = u[j - 32] + b3[j];
+        }
+        if (!publish_group(g, ok)) break;
         if (rows == kRows) {
             if (r == 0) bulk_store(z + kOut * row0, smem_addr(zs), kRows * kOut * 4);
         } else {
@@ -651,13 +663,12 @@ __global__ void __launch_bounds__(kInferGroups * kRows, 1) k_sur_infer(const Sur
             for (int k = 0; k < 6; ++k) f[k] = qs[r].x[k];
         }
         store_input_row(gs + S::X, r, f);
-        publish_group(g);
-        forward_tile<S>(sm, gs, tcol, t_row, phase, r, g, ok);
+        publish_group(g, true);
+        if (!forward_tile<S>(sm, gs, tcol, t_row, phase, r, g, ok)) break;
         float zz[kOutPad];
-        output_epilogue(t_row, b3, zz);
+        if (ok) output_epilogue(t_row, b3, zz);
         tc_fence_before();
-        ok = group_sync_and(g, ok);
-        if (!ok) break;
+        if (!group_sync_and(g, ok)) break;
 
         bool emit = false;
         PhaseRec rec;
@@ -931,12 +942,6 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_sur_train(const SurNet net
     const Operand w1K{s0 + S::Img + kImgW1, kInPad, false}, w2K{s0 + S::Img + kImgW2, kH, false},
         w3pK{s0 + S::W3P, kH, false};
     const Operand w2M{s0 + S::Img + kImgW2, kH, true}, w3M{s0 + S::Img + kImgW3, kH, true};
-    auto step = [&]() {                             // the tensor core's work committed last
-        const bool done = mbar_wait(bar, phase);
-        phase ^= 1u;
-        tc_fence_after();
-        return done;
-    };
     for (long long tile = blockIdx.x; first + tile * kRows < end; tile += gridDim.x) {
         const long long row = first + tile * kRows + r;
         const bool valid = row < end;
@@ -959,41 +964,37 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_sur_train(const SurNet net
             for (int j = 0; j < kDY; ++j) y[j] = __ldg(yt + 5 * row + j);
         }
         // ---- layer 1 (the CTA agrees here on the waits so far) ----
-        fence_async_smem();
-        tc_fence_before();
-        if (!__syncthreads_and(ok)) {
-            ok = false;
-            break;
-        }
+        if (!publish(ok)) break;
         if (threadIdx.x == 0) {
             tc_fence_after();
             mma_operands(tbase, xK, w1K, kInPad, kH, false);
             umma_commit(bar);
         }
-        ok = step() && ok;
-        const uint32_t m1 = hidden_epilogue_train(t_row, b1, sm + S::H1, kH1Cols, r, c0);
+        ok = work_done(bar, phase);
+        uint32_t m1 = 0u, m2 = 0u;
+        if (ok) m1 = hidden_epilogue_train(t_row, b1, sm + S::H1, kH1Cols, r, c0);
         // ---- layer 2 ----
-        publish();
+        if (!publish(ok)) break;
         if (threadIdx.x == 0) {
             tc_fence_after();
             mma_operands(tbase + 128u, h1K, w2K, kH, kH, false);
             umma_commit(bar);
         }
-        ok = step() && ok;
-        const uint32_t m2 = hidden_epilogue_train(t_row + 128u, b2, sm + S::H2, kH, r, c0);
+        ok = work_done(bar, phase);
+        if (ok) m2 = hidden_epilogue_train(t_row + 128u, b2, sm + S::H2, kH, r, c0);
         // ---- output layer: component cg's 16 columns ----
-        publish();
+        if (!publish(ok)) break;
         if (threadIdx.x == 0) {
             tc_fence_after();
             mma_operands(tbase, h2K, w3pK, kH, kOutP, false);
             umma_commit(bar);
         }
-        ok = step() && ok;
+        ok = work_done(bar, phase);
         // loss of the row and its gradient with respect to z (BCE of the
         // transmission logit plus, for transmitted tracks, the negative
         // log-likelihood of the mixture); this thread has component cg
-        float zv[16];
-        tmem_ld16(t_row + (uint32_t)(16 * cg), zv);
+        float zv[16] = {};
+        if (ok) tmem_ld16(t_row + (uint32_t)(16 * cg), zv);
 #pragma unroll
         for (int j = 0; j < 16; ++j) zv[j] += b3[16 * cg + j];
         const float alpha = zv[1];
@@ -1060,7 +1061,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_sur_train(const SurNet net
             *reinterpret_cast<unsigned short*>(sm + S::DZ + kmaj(r, col[j], kOutPad)) = bf16_bits(g[j]);
         }
         // ---- dh2 = dz W3 and dW3^T += h2^T dz ----
-        publish();
+        if (!publish(ok)) break;
         if (threadIdx.x == 0) {
             tc_fence_after();
             mma_operands(tbase, dzK, w3M, kOutPad, kH, false);
@@ -1072,11 +1073,11 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_sur_train(const SurNet net
             const float sum = warp_sum(g[j]);
             if (lane == 0 && (j > 0 || cg == 0)) s_red[kOutPad * q + col[j]] = sum;
         }
-        ok = step() && ok;
+        ok = work_done(bar, phase);
         // ---- da2 = dh2 * relu'(a2), over h2 ----
-        masked_epilogue(t_row, m2, sm + S::H2, r, c0);
+        if (ok) masked_epilogue(t_row, m2, sm + S::H2, r, c0);
         // ---- dh1 = da2 W2 and [dW2 | db2] += da2^T [h1 | 1] ----
-        publish();
+        if (!publish(ok)) break;
         if (threadIdx.x == 0) {
             tc_fence_after();
             mma_operands(tbase + 128u, h2K, w2M, kH, kH, false);
@@ -1089,17 +1090,17 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_sur_train(const SurNet net
             for (int k = 0; k < 4; ++k) d += s_red[kOutPad * k + threadIdx.x];
             s_db3[threadIdx.x] = (float)d;
         }
-        ok = step() && ok;
+        ok = work_done(bar, phase);
         // ---- da1 = dh1 * relu'(a1), over da2 ----
-        masked_epilogue(t_row + 128u, m1, sm + S::H2, r, c0);
+        if (ok) masked_epilogue(t_row + 128u, m1, sm + S::H2, r, c0);
         // ---- [dW1 | db1] += da1^T [x | 1] ----
-        publish();
+        if (!publish(ok)) break;
         if (threadIdx.x == 0) {
             tc_fence_after();
             mma_operands(tbase + kColW1, h2M, xM, kRows, kInPad, tiles_done > 0);
             umma_commit(bar);
         }
-        ok = step() && ok;
+        ok = work_done(bar, phase);
         ++tiles_done;
     }
     // ---- loss and the accumulated weight gradients ----
