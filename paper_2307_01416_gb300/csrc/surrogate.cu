@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(kFwdGroups * kRows, 1) k_sur_forward(const Sur
     const uint32_t t_row = tcol + ((uint32_t)((r >> 5) * 32) << 16);
     const uint32_t bar = smem_addr(gs + S::Bar), bar_in = bar + 8u;
     uint32_t phase = 0u, phase_in = 0u;
-    bool ok = true, loading = false;
+    bool ok = true, loading = false;                // loading: a copy of inputs was started and not seen complete
     float* xs = reinterpret_cast<float*>(gs + S::XS);
     float* zs = reinterpret_cast<float*>(gs + S::H);
     const float* b3 = reinterpret_cast<const float*>(sm + S::Bias) + 2 * kH;
@@ -551,18 +551,19 @@ __global__ void __launch_bounds__(kFwdGroups * kRows, 1) k_sur_forward(const Sur
         const int rows = (int)min((long long)kRows, n - row0);
         float f[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
         if (loading) {
-            ok = mbar_wait(bar_in, phase_in) && ok;
-            phase_in ^= 1u;
-            loading = false;
+            if (mbar_wait(bar_in, phase_in)) {
+                phase_in ^= 1u;
+                loading = false;
 #pragma unroll
-            for (int k = 0; k < 6; ++k) f[k] = xs[kIn * r + k];
+                for (int k = 0; k < 6; ++k) f[k] = xs[kIn * r + k];
+            }
         } else if (r < rows) {
 #pragma unroll
             for (int k = 0; k < 6; ++k) f[k] = __ldg(x + kIn * (row0 + r) + k);
         }
         store_input_row(gs + S::X, r, f);
         if (r == 0) bulk_store_wait_read();         // the last outputs have left the staging tile
-        if (!publish_group(g, ok)) break;
+        if (!publish_group(g, !loading)) break;
         loading = whole(tile + stride);
         if (loading && r == 0)
             bulk_load(smem_addr(xs), x + kIn * kRows * (tile + stride), kRows * kIn * 4, bar_in);
@@ -585,7 +586,10 @@ __global__ void __launch_bounds__(kFwdGroups * kRows, 1) k_sur_forward(const Sur
             for (int i = r; i < rows * kOut; i += kRows) z[kOut * row0 + i] = zs[i];
         }
     }
-    if (!ok && loading) (void)mbar_wait(bar_in, phase_in);     // a copy in flight ends before the memory is given back
+    if (loading) {                                  // the group stopped: its copy ends before the memory is given back
+        atomicOr(net.status, 1);
+        (void)mbar_wait(bar_in, phase_in);
+    }
     if (r == 0) bulk_store_wait();
     fwd_epilogue_free<S>(sm, tbase, bar, phase, ok, net);
 }
@@ -930,7 +934,8 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_sur_train(const SurNet net
     const uint32_t t_row = tbase + ((uint32_t)(q * 32) << 16);
     const int c0 = 32 * cg;
     uint32_t phase = 0u;
-    bool ok = mbar_wait(bar_img, 0u);
+    const bool images = mbar_wait(bar_img, 0u);
+    bool ok = true;
     int tiles_done = 0;
     double loss_acc = 0.0;
     const long long end = min(first + rows, n);
@@ -964,7 +969,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_sur_train(const SurNet net
             for (int j = 0; j < kDY; ++j) y[j] = __ldg(yt + 5 * row + j);
         }
         // ---- layer 1 (the CTA agrees here on the waits so far) ----
-        if (!publish(ok)) break;
+        if (!publish(ok && images)) break;
         if (threadIdx.x == 0) {
             tc_fence_after();
             mma_operands(tbase, xK, w1K, kInPad, kH, false);
@@ -1111,7 +1116,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_sur_train(const SurNet net
     // the CTA's partial gradient, every parameter written once (plain stores;
     // the Adam step sums the CTAs' partials: no contended atomics)
     float* part = net.gpart + (long long)blockIdx.x * kNParams;
-    const bool have = __syncthreads_and(ok) && tiles_done > 0;
+    const bool have = __syncthreads_and(ok && images) && tiles_done > 0;
     {
         const int h = r;
         store_partial<32>(t_row + kColW2 + (uint32_t)c0, have, part + oW2 + h * kH + c0);
@@ -1137,9 +1142,10 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_sur_train(const SurNet net
         }
         if (threadIdx.x < kOut) part[ob3 + threadIdx.x] = have ? s_db3[threadIdx.x] : 0.0f;
     }
-    if (!ok) {                                      // a wait failed in this thread
+    if (!ok || !images) {                           // a wait failed here: what it waited for ends before the CTA does
         atomicOr(net.status, 1);
-        (void)mbar_wait(bar, phase);
+        if (!ok) (void)mbar_wait(bar, phase);
+        if (!images) (void)mbar_wait(bar_img, 0u);
     }
     tc_fence_before();
     __syncthreads();

@@ -150,3 +150,20 @@ def test_training_stops_at_a_failed_wait(run, thread):
         r = run("train", 256, thread, call)
         assert r["status"] == 1 and r["gradient"] == 0
         assert r["waits"] == clean["waits"][:call + 1] + [clean["waits"][call]]
+
+
+@pytest.mark.parametrize("thread", [0, 77, 127])
+def test_copies_in_flight_are_waited_for(run, thread):
+    """A bulk copy whose wait failed, or that was started for a tile that is
+    not begun any more, is waited for once more; no GEMM is begun without it."""
+    clean = run("forward", 128, thread, -1)
+    r = run("forward", 128, thread, 0)
+    assert r["status"] == 1 and r["tiles"] == [0] and r["waits"] == 2 * clean["waits"][:1]
+    # the first GEMM fails while the pipeline's next inputs are on their way
+    r = run("forward", 10 * 128, thread, 1)
+    inputs, gemm = clean["waits"][:2]
+    assert r["status"] == 1 and r["tiles"] == [0 if t % 4 == 0 else 45 * 128 for t in range(10)]
+    assert r["waits"][:2] == [inputs, gemm] and sorted(r["waits"][2:]) == sorted([(inputs[0], 1 - inputs[1]), gemm])
+    clean = run("train", 256, thread, -1)
+    r = run("train", 256, thread, 0)
+    assert r["status"] == 1 and r["gradient"] == 0 and r["waits"] == 2 * clean["waits"][:1]
