@@ -396,7 +396,9 @@ typedef struct {
  * optimised weights out.  history: optional host float [iterations], the
  * worst-case objective before each step.  ms: optional host float [2]: device
  * time of the iterations, then of the setup (CUDA events).  stream: a
- * cudaStream_t (NULL = legacy default).
+ * cudaStream_t (NULL = legacy default); any other stream first waits for what
+ * the legacy default stream has been given so far, so inputs made there are
+ * complete (the two calls below as well).
  * Only target and ring voxels enter the objective, so the call first copies
  * their rows of every matrix into a compact form (scratch of about 6 bytes
  * per such entry, allocated and freed by the call), then iterates on those.

@@ -1831,6 +1831,22 @@ vpmc_status check_opt_inputs(const vpmc_csr* mats, int n_scen, const uint8_t* cl
     return VPMC_OK;
 }
 
+// Makes `stream` wait for what the legacy default stream has been given so far
+// (and, as work on that stream does, for the blocking streams' work): a caller
+// may pass a stream of its own for matrices, classes and weights that were made
+// on the default one.
+cudaError_t wait_default_stream(cudaStream_t stream)
+{
+    if (stream == nullptr || stream == cudaStreamLegacy) return cudaSuccess;
+    cudaEvent_t made = nullptr;
+    cudaError_t e = cudaEventCreateWithFlags(&made, cudaEventDisableTiming);
+    if (e != cudaSuccess) return e;
+    e = cudaEventRecord(made, cudaStreamLegacy);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, made, 0);
+    cudaEventDestroy(made);
+    return e;
+}
+
 int current_sms()
 {
     int dev = 0, sms = 0;
@@ -1855,6 +1871,7 @@ vpmc_status vpmc_robust_optimize(const vpmc_csr* mats, int n_scen, const uint8_t
     OptInputs in;
     vpmc_status st = check_opt_inputs(mats, n_scen, voxel_class_dev, &in);
     if (st != VPMC_OK) return st;
+    CUDA_TRY(wait_default_stream((cudaStream_t)stream));
     OptSpec spec;
     ClassRows* rows = nullptr;
     struct RowsFree {
@@ -1898,6 +1915,7 @@ vpmc_status vpmc_weights_dose(const vpmc_csr* mat, const float* x_dev, float* do
     if (!mat || !x_dev || !dose_dev || !mat->row_ptr || mat->n_rows <= 0 || mat->n_cols <= 0 ||
         mat->n_cols > INT32_MAX || (mat->nnz > 0 && (!mat->col || !mat->val)))
         return fail(VPMC_ERR_ARG, "bad argument");
+    CUDA_TRY(wait_default_stream((cudaStream_t)stream));
     CUDA_TRY(run_weights_dose(reinterpret_cast<const long long*>(mat->row_ptr), mat->col, mat->val, mat->n_rows,
                               (int)mat->n_cols, x_dev, dose_dev, (cudaStream_t)stream, current_sms()));
     return VPMC_OK;
@@ -1912,6 +1930,7 @@ vpmc_status vpmc_target_indices(const vpmc_csr* mats, int n_scen, const uint8_t*
     OptInputs in;
     vpmc_status st = check_opt_inputs(mats, n_scen, voxel_class_dev, &in);
     if (st != VPMC_OK) return st;
+    CUDA_TRY(wait_default_stream((cudaStream_t)stream));
     CUDA_TRY(run_target_indices(in.rp.data(), in.col.data(), in.val.data(), n_scen, in.n_rows, in.n_cols,
                                 voxel_class_dev, prescription, x_dev, out, (cudaStream_t)stream, current_sms()));
     return VPMC_OK;
