@@ -18,7 +18,7 @@ namespace vpmc {
 // every workload measured, or within 1 % of it (k_patient on 3.2e7 histories in
 // the head: 121.6 ms at 896 threads, 123.5 at 768, 136.9 at 512; aggregated
 // atomics 219.9 ms; chunks of 128 122.2 ms there and 4.3 against 3.8 ms on 4e6
-// histories behind an aperture; chunks of 16 a third slower in the beam-line
+// histories behind an aperture; chunks of 16 within 1 % in the beam-line
 // kernels), so nothing is timed before a context's first call.
 struct LaunchShape {
     int dev_block = 768;     // k_aperture threads per block (a full block)
