@@ -169,15 +169,24 @@ uint32_t local_edges(const double* xy, int n, double x0, double y0, double x1, d
         if (std::max(ya, yb) < y0 || std::min(ya, yb) > y1 || std::max(xa, xb) < x0) kind[i] = kOut;
         else kind[i] = std::min(xa, xb) > x1 ? kRight : kEval;
     }
-    // edge i ends in vertex i, edge i + 1 starts there
-    for (bool grew = true; grew;) {
+    // edge i ends in vertex i, edge i + 1 starts there.  What an edge hands on
+    // goes round the polygon one way: two rounds each way reach all of it (a
+    // thin slot of 4,096 vertices, half of whose edges meet in one cell's
+    // height: 2.4 s a raster with rounds until nothing changed, 0.4 s)
+    auto hand_on = [&](int from, int to, int v) {
+        if (kind[to] != kRight || kind[from] == kRight || xy[2 * v + 1] < y0 || xy[2 * v + 1] > y1) return false;
+        kind[to] = kEval;
+        return true;
+    };
+    bool grew = true;
+    for (int round = 0; round < 2 && grew; ++round) {
         grew = false;
-        for (int i = 0; i < n; ++i) {
-            const int j = (i + 1) % n;
-            if (Y(i) < y0 || Y(i) > y1 || (kind[i] != kRight && kind[j] != kRight) || kind[i] == kind[j]) continue;
-            kind[kind[i] == kRight ? i : j] = kEval;
-            grew = true;
-        }
+        for (int i = 0; i < n; ++i) grew |= hand_on(i, i + 1 < n ? i + 1 : 0, i);
+    }
+    grew = true;
+    for (int round = 0; round < 2 && grew; ++round) {
+        grew = false;
+        for (int i = n - 1; i >= 0; --i) grew |= hand_on(i + 1 < n ? i + 1 : 0, i, i);
     }
     int first = -1, last = -1, gap = 0, start = 0;
     for (int i = 0; i < n; ++i) {
