@@ -1314,7 +1314,7 @@ vpmc_status vpmc_influence_matrix(vpmc_ctx* c, const vpmc_spot* spots, int n_spo
         // column maxima over boxes, then bucket the out-of-box records and raise the maxima
         IM_TRY(ensure(c->im_colmax, items.size(), &d_colmax));
         IM_TRY(launch_column_max(c->d_scratch, c->d_items, c->d_boxes, c->d_inv_rho, c->d_inv_rho_f, c->sg, 0,
-                                 (int)items.size(), d_colmax, c->stream));
+                                 (int)items.size(), d_colmax, c->num_sms, c->stream));
         ++c->launches;
         const long long n_buckets = (long long)ns * c->nvox;
         if (n_ovf) {

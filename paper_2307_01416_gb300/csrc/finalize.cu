@@ -493,16 +493,17 @@ cudaError_t launch_dose_normalise(const unsigned long long* acc, const double* r
     return cudaGetLastError();
 }
 
-constexpr int kColumnMaxBlocks = 152 * 16;
+constexpr int kColumnMaxBlocks = 16;             // per SM
 
 cudaError_t launch_column_max(const unsigned long long* scratch, const DevItem* items, const DevBox* boxes,
                               const double* inv_rho, const float* inv_rho_f, const Grid3 sg, int first_item,
-                              int n_items, double* colmax, cudaStream_t s)
+                              int n_items, double* colmax, int num_sms, cudaStream_t s)
 {
     if (n_items <= 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(colmax, 0, (size_t)n_items * sizeof(double), s);
     if (e != cudaSuccess) return e;
-    const int split = n_items < kColumnMaxBlocks ? (kColumnMaxBlocks + n_items - 1) / n_items : 1;
+    const int blocks = num_sms * kColumnMaxBlocks;
+    const int split = n_items < blocks ? (blocks + n_items - 1) / n_items : 1;
     k_column_max<<<dim3((unsigned)n_items, (unsigned)split), 512, 0, s>>>(scratch, items, boxes, inv_rho, inv_rho_f, sg, first_item, colmax);
     return cudaGetLastError();
 }

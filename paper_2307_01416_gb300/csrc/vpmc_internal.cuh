@@ -424,7 +424,7 @@ cudaError_t launch_dose_normalise(const unsigned long long* acc, const double* r
 // inv_rho_f: the same in FP32, for the screen).
 cudaError_t launch_column_max(const unsigned long long* scratch, const DevItem* items, const DevBox* boxes,
                               const double* inv_rho, const float* inv_rho_f, const Grid3 sg, int first_item,
-                              int n_items, double* colmax, cudaStream_t s);
+                              int n_items, double* colmax, int num_sms, cudaStream_t s);
 // out = 1 / x in FP64, out_f its FP32 value.
 cudaError_t launch_reciprocal(const double* x, long long n, double* out, float* out_f, cudaStream_t s);
 
