@@ -43,14 +43,19 @@ using namespace dev;
 using namespace tr;
 
 constexpr int kModeAllPhysics = 1;   // scattering, straggling and nuclear removal on
-constexpr int kModeIMScoring = 2;    // unit item weights, fx32, plain atomics
+constexpr int kModeIMScoring = 2;    // unit item weights, fx32, plain atomics, at most kMax32BitSteps steps
+
+// Steps of a history whose fixed-point total fits 32 bits: 250 MeV at 2^24 are
+// 4,194,304,000, and each step adds at most half a unit of the deposit's
+// rounding and 128 units of the energy's (half an ulp of a binary32 below
+// 256): 2^19 steps stay below 2^32.
+constexpr int kMax32BitSteps = 1 << 19;
 
 template <int kNest, int kMode>
 __global__ void __launch_bounds__(kPatientMaxBlock, 1) k_patient(const TransportParams P)
 {
     constexpr bool kIM = (kMode & kModeIMScoring) != 0;
-    // a history's fixed-point total: at 2^24 and below, 250 MeV and every
-    // rounding of its steps stay below 2^32
+    // a history's fixed-point total (32 bits: see kMax32BitSteps)
     using DepT = std::conditional_t<kIM, unsigned, unsigned long long>;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
@@ -368,7 +373,8 @@ template <int kNest>
 cudaError_t launch_patient_nest(const TransportParams& p, int grid, int block, cudaStream_t s)
 {
     if (!(p.mcs && p.straggling && p.nuclear)) return launch_patient_variant<kNest, 0>(p, grid, block, s);
-    if (p.unit_weight && p.fx32 && !p.aggregate)
+    // (a longer iteration cap takes the variant with 64-bit totals)
+    if (p.unit_weight && p.fx32 && !p.aggregate && p.max_iter <= kMax32BitSteps)
         return launch_patient_variant<kNest, kModeAllPhysics | kModeIMScoring>(p, grid, block, s);
     return launch_patient_variant<kNest, kModeAllPhysics>(p, grid, block, s);
 }
