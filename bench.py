@@ -390,7 +390,7 @@ def main():
                             "spot) column boxes cut at each energy layer's reach along its field, zeroed, scanned for "
                             "column maxima, then read by the count and fill passes of the CSR; deposits beyond a box "
                             "are out-of-box records, merged into the CSR"}
-        adds_rate = patient_steps / (ms_patient / 1000.0) if ms_patient > 0 else None
+        steps_rate = patient_steps / (ms_patient / 1000.0) if ms_patient > 0 else None
         roof = {"bound": "alu", "achieved": achieved, "peak": peak_tops, "unit": "Tops/s",
                 "frac": achieved / peak_tops, "traffic": traffic, "kernel": "k_source_rs+k_aperture+k_patient",
                 "peak_note": "%d SMs x 4 sub-partitions x 32 lanes x %.0f MHz (max SM clock) lane-ops/s; "
@@ -399,12 +399,11 @@ def main():
                 "kernel_ms_per_step": kern_ms / args.steps, "steps_per_launch": steps / args.steps,
                 "ops_per_step": ops / max(steps, 1),
                 "l2_atomic": {"kernel": "k_patient", "unit": "adds/s",
-                              "achieved": adds_rate, "peak": l2["adds_per_s"],
-                              "frac": adds_rate / l2["adds_per_s"] if adds_rate else None,
+                              "steps_per_s": steps_rate, "peak": l2["adds_per_s"],
                               "k_patient_ms_per_step": ms_patient / args.steps,
-                              "note": "upper bound: one 64-bit scoring add per patient step (the kernel adds once "
-                                      "per voxel visit) over k_patient's CUDA-event time; peak = "
-                                      "vpmc_measure_l2_atomics over a 32 MiB buffer"}}
+                              "note": "steps_per_s bounds the kernel's 64-bit scoring adds from above: one per voxel "
+                                      "visit, about a third of its steps; peak = vpmc_measure_l2_atomics over a "
+                                      "32 MiB buffer"}}
         e2e = _leg(lambda: e2e_leg(pb, spots, scens, opts, args), not args.no_e2e)
         cpu = _leg(lambda: cpu_baseline(pb, spots, args.cpu_seconds), not args.no_cpu_baseline and world == 1)
         opt = _leg(lambda: optimizer_leg(pb, target, last_mats, args), not args.no_optimizer and world == 1)

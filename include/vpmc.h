@@ -217,7 +217,12 @@ vpmc_status vpmc_set_aperture(vpmc_ctx* ctx, int beam_id, const vpmc_beam* beam)
  * that error without running (the earlier call's dose is then not valid).
  * Spot errors: VPMC_ERR_STATE for a beam id that was not set,
  * VPMC_ERR_ARG for an energy outside (0.5, 250] MeV (NaN included), n_hist
- * outside [0, 2^32), a negative or non-finite sigma, divergence or weight. */
+ * outside [0, 2^32), a negative or non-finite sigma, divergence or weight.
+ * dose_dev is written as a whole at the end of the call's work (also without
+ * histories) and not before: a call that is refused or fails on the way
+ * leaves it as it was; after
+ * VPMC_ERR_TIMEOUT or VPMC_ERR_DEVICE_FLAG it holds the dose of the histories
+ * that were transported. */
 vpmc_status vpmc_run_spots(vpmc_ctx* ctx, const vpmc_spot* spots, int n_spots, const vpmc_scenario* scen,
                            const vpmc_opts* opts, float* dose_dev, vpmc_stats* stats_out);
 
@@ -426,8 +431,8 @@ vpmc_status vpmc_target_indices(const vpmc_csr* mats, int n_scen, const uint8_t*
  * ------------------------------------------------------------------------ */
 
 /* The current device's rate of 64-bit atomic adds resolved in L2: the
- * secondary bound of the transport's scoring, which adds each
- * condensed-history step's fixed-point deposit to a voxel with one such add.
+ * secondary bound of the transport's scoring, which adds the fixed-point
+ * deposits of each visit of a voxel to it with one such add.
  * 4 x SMs blocks of 1024 threads each make `iters` adds of 1 to entries of a
  * device buffer of n_entries 64-bit words (a power of two in [32, 2^26];
  * 2^22 words, 32 MiB, stay in L2), chosen by a hash of (thread, iteration),

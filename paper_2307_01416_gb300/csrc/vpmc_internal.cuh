@@ -307,7 +307,6 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned block, size_t
     return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
-// Host-side launchers (transport.cu, finalize.cu).
 // Threads per block of a persistent launch over at most n histories: warps that
 // the work cannot fill are left out, so that every SM gets some of it.  With
 // full blocks the first ones to have staged their tables take all of a small
@@ -344,6 +343,7 @@ inline void beam_flags(TransportParams* p, const DevBeam* beams, int n)
     }
 }
 
+// Host-side launchers (devices.cu, patient.cu, finalize.cu).
 // Transport of histories [p.hist_begin, p.total): the beam-line kernels
 // (source and range shifter, then the aperture: launch_devices), then the
 // patient kernel on the histories they hand over (p.mid and p.phase must each hold p.total - p.hist_begin records).
