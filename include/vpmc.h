@@ -220,9 +220,8 @@ vpmc_status vpmc_set_aperture(vpmc_ctx* ctx, int beam_id, const vpmc_beam* beam)
  * outside [0, 2^32), a negative or non-finite sigma, divergence or weight.
  * dose_dev is written as a whole at the end of the call's work (also without
  * histories) and not before: a call that is refused or fails on the way
- * leaves it as it was; after
- * VPMC_ERR_TIMEOUT or VPMC_ERR_DEVICE_FLAG it holds the dose of the histories
- * that were transported. */
+ * leaves it as it was; after VPMC_ERR_TIMEOUT or VPMC_ERR_DEVICE_FLAG it holds
+ * the dose of the histories that were transported. */
 vpmc_status vpmc_run_spots(vpmc_ctx* ctx, const vpmc_spot* spots, int n_spots, const vpmc_scenario* scen,
                            const vpmc_opts* opts, float* dose_dev, vpmc_stats* stats_out);
 

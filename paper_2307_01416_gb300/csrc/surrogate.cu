@@ -792,7 +792,7 @@ __global__ void __launch_bounds__(kInferGroups * kRows, 1) k_sur_infer(const Sur
 // 4-way bank conflicts); the b3 gradient by one butterfly per component.
 // 20.7 us a launch; 40.8 us with 128 threads and transposed copies.  The Adam
 // step and the next launch start while their predecessor drains (their own
-// set-up runs meanwhile): 33 -> 28.6 us a training step; 28.8 with the vote on
+// set-up runs meanwhile): 33 -> 28.6 us a training step; 29.0 with the vote on
 // the waits in the barrier before each product.
 constexpr int kTrainThreads = 512;
 constexpr int kH1Cols = kH + 16;             // h1 and the all-ones column (b2 gradient)
